@@ -11,7 +11,7 @@
 // adj(J) / det J.  For the brick the natural derivatives are tensor products of
 // the 1D hat functions, so the map from the 8 x 6 values of M_q to the 36
 // packed entries factorises along the three axes (sum factorisation): about
-// 1.2 kflop per element instead of about 3.8 kflop for forming B and B^T B
+// 1 kflop per element instead of about 3.8 kflop for forming B and B^T B
 // point by point.  J_q itself is a bilinear interpolation of the 4 element edges
 // along each axis, formed from coordinate differences so that FP32 keeps its
 // accuracy relative to the element size.
@@ -19,6 +19,8 @@
 
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include "pair.cuh"
 
 namespace fem {
 
@@ -200,53 +202,6 @@ __device__ __forceinline__ void brick_jrows(const Vec3<T> (&e)[3][2][2], Vec3<T>
     }
 }
 
-// M_q (times 2, see brick_ke) for the 8 Gauss points q = 4 q1 + 2 q2 + q3, as
-// (rr, ss, tt, rs, rt, st), times the factor s (the element's c / 8, applied
-// once per point instead of once per packed entry); det[q] = det(2 J_q).
-template <typename T>
-__device__ __forceinline__ void brick_M(const Vec3<T> (&row)[3][2][2], T s, T (&M)[8][6], T (&det)[8]) {
-#pragma unroll
-    for (int q1 = 0; q1 < 2; ++q1)
-#pragma unroll
-        for (int q2 = 0; q2 < 2; ++q2)
-#pragma unroll
-            for (int q3 = 0; q3 < 2; ++q3) {
-                const int q = 4 * q1 + 2 * q2 + q3;
-                const Vec3<T> &R = row[0][q2][q3];
-                const Vec3<T> &S = row[1][q1][q3];
-                const Vec3<T> &U = row[2][q1][q2];
-                const Vec3<T> C0 = cross3(S, U), C1 = cross3(U, R), C2 = cross3(R, S);
-                const T d = dot3(R, C0);
-                det[q] = d;
-                const T inv = rcp_rn(d < T(0) ? -d : d) * s;
-                M[q][0] = dot3(C0, C0) * inv;
-                M[q][1] = dot3(C1, C1) * inv;
-                M[q][2] = dot3(C2, C2) * inv;
-                M[q][3] = dot3(C0, C1) * inv;
-                M[q][4] = dot3(C0, C2) * inv;
-                M[q][5] = dot3(C1, C2) * inv;
-            }
-}
-
-// T[c][d] = sum_{u,v} A[u][v] F_c(u) F_d(v), F_0 = (PP, QQ), F_1 = (QQ, PP), F_2 = (PQ, PQ).
-template <typename T>
-__device__ __forceinline__ void contract_FF(const T (&A)[2][2], T (&out)[3][3]) {
-    const T PP = T(FEM_GPP), QQ = T(FEM_GQQ), PQ = T(FEM_GPQ);
-    T U[2][3];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        U[u][0] = PP * A[u][0] + QQ * A[u][1];
-        U[u][1] = QQ * A[u][0] + PP * A[u][1];
-        U[u][2] = PQ * (A[u][0] + A[u][1]);
-    }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        out[0][d] = PP * U[0][d] + QQ * U[1][d];
-        out[1][d] = QQ * U[0][d] + PP * U[1][d];
-        out[2][d] = PQ * (U[0][d] + U[1][d]);
-    }
-}
-
 // Contract one Gauss axis of m[8] (index 4 q1 + 2 q2 + q3) with the hats
 // (kind 0: phi_x, 2 outputs) or the hat products (kind 1: F_c, 3 outputs).
 // The cross terms need V[x or c][y or c][z or c] over the three axes in turn.
@@ -298,71 +253,384 @@ __device__ __forceinline__ void contract_cross(const T (&m)[2][2][2], T (&V)[3][
     (void)N1;
 }
 
-// Packed lower k_e (36 entries, p = a(a+1)/2 + b) from the M_q of brick_M.
-// With J~ = 2J and dN~ = 2 dN (signs instead of +-1/2), M = M~/2 and
-// k_ab = (c / 8) sum_q dN~_a^T M~_q dN~_b; the factor c / 8 comes in M (brick_M).
+// ------------------------------------------------------ brick stiffness, in pairs
+// The brick's arithmetic runs on pairs (pair.cuh): every quantity that depends on
+// the Gauss point index q1 is held for q1 = 0 and 1 together, so FP32 needs one
+// packed instruction for two points.  Only the 1D operators along axis 1 itself
+// work inside a pair, in scalars.  The build kernels are bound by latency at 16
+// warps an SM, so an element's shorter instruction stream pays less than its count:
+// 1M bricks 236 -> 228 us mixed (512 meshes in one launch 3.30 -> 3.17 ms), with
+// the FP32 result's error against 64 bits 1.1e-7 -> 0.7e-7; FP64, whose pipe is
+// busy throughout, 2.41 -> 2.26 ms from the shared sums alone.
+
+// Rows of 2 J_q at the Gauss points: R (axis 1) does not depend on q1, S (axis 2)
+// and U (axis 3) hold q1 = 0 and 1 as pairs: R[q2][q3], S[q3], U[q2].
 template <typename T>
-__device__ __forceinline__ void brick_contract(const T (&M)[8][6], T (&k)[36]) {
-    T Arr[2][2], Ass[2][2], Att[2][2];
-    T mrs[2][2][2], mrt[2][2][2], mst[2][2][2];
+struct BrickRows {
+    Vec3<T> R[2][2];
+    Vec3<Pair<T>> S[2], U[2];
+};
+
+// Edges (differences formed in S, rounded once to T): r[i][j] along axis 1 at bits
+// (i, j) of axes 2 and 3; s[j], u[j] along axes 2 and 3 as pairs over the bit of
+// axis 1, at bit j of axis 3 and 2.
+template <typename T, typename S>
+__device__ __forceinline__ void brick_edge_pairs(const S (*xc)[3], int k, T (&r)[2][2], Pair<T> (&s)[2],
+                                                 Pair<T> (&u)[2]) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u)
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int v = 0; v < 2; ++v) {
-            Arr[u][v] = M[0 + 2 * u + v][0] + M[4 + 2 * u + v][0];      // sum over q1
-            Ass[u][v] = M[4 * u + 0 + v][1] + M[4 * u + 2 + v][1];      // sum over q2
-            Att[u][v] = M[4 * u + 2 * v + 0][2] + M[4 * u + 2 * v + 1][2];  // sum over q3
+        for (int j = 0; j < 2; ++j) r[i][j] = T(xc[hnode(1, i, j)][k] - xc[hnode(0, i, j)][k]);
+    if constexpr (sizeof(S) == sizeof(T)) {
+        Pair<T> x[2][2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 2; ++j) x[i][j] = pair(xc[hnode(0, i, j)][k], xc[hnode(1, i, j)][k]);
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            s[j] = x[1][j] - x[0][j];
+            u[j] = x[j][1] - x[j][0];
         }
+    } else {
 #pragma unroll
-    for (int q1 = 0; q1 < 2; ++q1)
-#pragma unroll
-        for (int q2 = 0; q2 < 2; ++q2)
-#pragma unroll
-            for (int q3 = 0; q3 < 2; ++q3) {
-                const int q = 4 * q1 + 2 * q2 + q3;
-                mrs[q1][q2][q3] = M[q][3];
-                mrt[q1][q2][q3] = M[q][4];
-                mst[q1][q2][q3] = M[q][5];
-            }
-    T Trr[3][3], Tss[3][3], Ttt[3][3];
-    contract_FF(Arr, Trr);  // [c2][c3]
-    contract_FF(Ass, Tss);  // [c1][c3]
-    contract_FF(Att, Ttt);  // [c1][c2]
-    T Vrs[3][3][3], Vrt[3][3][3], Vst[3][3][3];
-    contract_cross<T, 0, 0, 1>(mrs, Vrs);  // [x][y][c3]
-    contract_cross<T, 0, 1, 0>(mrt, Vrt);  // [x][c2][z]
-    contract_cross<T, 1, 0, 0>(mst, Vst);  // [c1][y][z]
-#pragma unroll
-    for (int a = 0; a < 8; ++a) {
-#pragma unroll
-        for (int b = 0; b <= a; ++b) {
-            const int a1 = hb1(a), a2 = hb2(a), a3 = hb3(a);
-            const int b1 = hb1(b), b2 = hb2(b), b3 = hb3(b);
-            const int c1 = hcls(a1, b1), c2 = hcls(a2, b2), c3 = hcls(a3, b3);
-            T v = T(hsig(a1) * hsig(b1)) * Trr[c2][c3];
-            v += T(hsig(a2) * hsig(b2)) * Tss[c1][c3];
-            v += T(hsig(a3) * hsig(b3)) * Ttt[c1][c2];
-            v += T(hsig(a1) * hsig(b2)) * Vrs[b1][a2][c3];
-            v += T(hsig(a2) * hsig(b1)) * Vrs[a1][b2][c3];
-            v += T(hsig(a1) * hsig(b3)) * Vrt[b1][c2][a3];
-            v += T(hsig(a3) * hsig(b1)) * Vrt[a1][c2][b3];
-            v += T(hsig(a2) * hsig(b3)) * Vst[c1][b2][a3];
-            v += T(hsig(a3) * hsig(b2)) * Vst[c1][a2][b3];
-            k[a * (a + 1) / 2 + b] = v;
+        for (int j = 0; j < 2; ++j) {
+            s[j] = pair(T(xc[hnode(0, 1, j)][k] - xc[hnode(0, 0, j)][k]),
+                        T(xc[hnode(1, 1, j)][k] - xc[hnode(1, 0, j)][k]));
+            u[j] = pair(T(xc[hnode(0, j, 1)][k] - xc[hnode(0, j, 0)][k]),
+                        T(xc[hnode(1, j, 1)][k] - xc[hnode(1, j, 0)][k]));
         }
     }
+}
+
+// hat_pair elementwise, and along axis 1 inside a pair.
+template <typename T>
+__device__ __forceinline__ void hat_pair(Pair<T> a, Pair<T> b, Pair<T> &o0, Pair<T> &o1) {
+    const Pair<T> d = a - b;
+    o0 = pfma(pair(T(FEM_GP), T(FEM_GP)), d, b);
+    o1 = pfma(pair(-T(FEM_GP), -T(FEM_GP)), d, a);
+}
+template <typename T>
+__device__ __forceinline__ Pair<T> hat_in_pair(Pair<T> p) {
+    T o0, o1;
+    hat_pair(pair_lo(p), pair_hi(p), o0, o1);
+    return pair(o0, o1);
+}
+
+template <typename T>
+__device__ __forceinline__ void brick_rows_k(const T (&r)[2][2], const Pair<T> (&s)[2], const Pair<T> (&u)[2],
+                                             T (&R)[2][2], Pair<T> (&So)[2], Pair<T> (&Uo)[2]) {
+    T m[2][2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) hat_pair(r[i][0], r[i][1], m[i][0], m[i][1]);
+#pragma unroll
+    for (int v = 0; v < 2; ++v) hat_pair(m[0][v], m[1][v], R[0][v], R[1][v]);
+    Pair<T> a, b;
+    hat_pair(s[0], s[1], a, b);
+    So[0] = hat_in_pair(a), So[1] = hat_in_pair(b);
+    hat_pair(u[0], u[1], a, b);
+    Uo[0] = hat_in_pair(a), Uo[1] = hat_in_pair(b);
+}
+
+template <typename T, typename S>
+__device__ __forceinline__ void brick_rows(const S (*xc)[3], BrickRows<T> &o) {
+    T r[2][2], R[2][2];
+    Pair<T> s[2], u[2], So[2], Uo[2];
+#define FEM_BRICK_ROWS(k, c)                          \
+    brick_edge_pairs<T, S>(xc, k, r, s, u);           \
+    brick_rows_k(r, s, u, R, So, Uo);                 \
+    o.R[0][0].c = R[0][0], o.R[0][1].c = R[0][1], o.R[1][0].c = R[1][0], o.R[1][1].c = R[1][1]; \
+    o.S[0].c = So[0], o.S[1].c = So[1], o.U[0].c = Uo[0], o.U[1].c = Uo[1];
+    FEM_BRICK_ROWS(0, x)
+    FEM_BRICK_ROWS(1, y)
+    FEM_BRICK_ROWS(2, z)
+#undef FEM_BRICK_ROWS
+}
+
+// a x b of pairs, given na = -a (packed instructions have no free negation).
+template <typename T>
+__device__ __forceinline__ Vec3<Pair<T>> cross3(const Vec3<Pair<T>> &a, const Vec3<Pair<T>> &na,
+                                                const Vec3<Pair<T>> &b) {
+    return {pfma(a.y, b.z, na.z * b.y), pfma(a.z, b.x, na.x * b.z), pfma(a.x, b.y, na.y * b.x)};
+}
+template <typename T>
+__device__ __forceinline__ Pair<T> dot3(const Vec3<Pair<T>> &a, const Vec3<Pair<T>> &b) {
+    return pfma(a.z, b.z, pfma(a.y, b.y, a.x * b.x));
+}
+template <typename T>
+__device__ __forceinline__ Vec3<Pair<T>> neg3(const Vec3<Pair<T>> &a) {
+    return {-a.x, -a.y, -a.z};
+}
+template <typename T>
+__device__ __forceinline__ Vec3<Pair<T>> both3(const Vec3<T> &a) {
+    return {pair(a.x, a.x), pair(a.y, a.y), pair(a.z, a.z)};
+}
+
+// 1 / |d| of both halves, as rcp_rn.  The FP32 form iterates on -1/|d|, whose sign
+// makes the residual 1 - |d| r a plain packed FMA, and returns -1/|d|.
+__device__ __forceinline__ Pair<float> neg_rcp_abs(Pair<float> d) {
+    const float x0 = fabsf(pair_lo(d)), x1 = fabsf(pair_hi(d));
+    float n0, n1;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(n0) : "f"(-x0));
+    asm("rcp.approx.f32 %0, %1;" : "=f"(n1) : "f"(-x1));
+    const Pair<float> n = pair(n0, n1);
+    return pfma(n, pfma(pair(x0, x1), n, pair(1.f, 1.f)), n);
+}
+__device__ __forceinline__ Pair<double> neg_rcp_abs(Pair<double> d) {
+    return {-rcp_rn(fabs(d.x)), -rcp_rn(fabs(d.y))};
+}
+
+// The hat products along one axis are taken six times over: 6 F_0 = (2 + g3, 2 - g3),
+// 6 F_1 = (2 - g3, 2 + g3), 6 F_2 = (1, 1) with g3 = sqrt(3), so that a contraction
+// is 2 (a + b) +- g3 (a - b) and a + b, five operations instead of six.  The
+// diagonal terms pass two such contractions and the cross terms one: their M_q are
+// scaled by 1/36 and 1/6.
+#define FEM_G3 1.7320508075688772935
+template <typename T>
+__device__ __forceinline__ void prod6(T a, T b, T &o0, T &o1, T &o2) {
+    o2 = a + b;
+    const T t = T(FEM_G3) * (a - b);
+    o0 = fma(T(2), o2, t);
+    o1 = fma(T(2), o2, -t);
+}
+template <typename T>
+__device__ __forceinline__ void prod6(Pair<T> a, Pair<T> b, Pair<T> (&o)[3]) {
+    const Pair<T> d = a - b;
+    o[2] = a + b;
+    const Pair<T> s = o[2] + o[2];
+    o[0] = pfma(pair(T(FEM_G3), T(FEM_G3)), d, s);
+    o[1] = pfma(pair(-T(FEM_G3), -T(FEM_G3)), d, s);
+}
+
+// M~_q = cof(2J_q) cof(2J_q)^T / |det 2J_q| (k_e = c/8 sum_q dN~_a^T M~_q dN~_b with
+// dN~ = 2 dN = +-1 times hats) as pairs over q1: M[q2][q3] holds (rr, ss, tt)
+// scaled by s/36 and (rs, rt, st) scaled by s/6; det = det(2 J_q).
+template <typename T>
+__device__ __forceinline__ void brick_M(const BrickRows<T> &row, T s, Pair<T> (&M)[2][2][6], Pair<T> (&det)[2][2]) {
+    const T sd = s * T(-1.0 / 36.0), sc = s * T(-1.0 / 6.0);
+    const Pair<T> wd = pair(sd, sd), wc = pair(sc, sc);
+    Vec3<Pair<T>> nU[2];
+#pragma unroll
+    for (int q2 = 0; q2 < 2; ++q2) nU[q2] = neg3(row.U[q2]);
+#pragma unroll
+    for (int q3 = 0; q3 < 2; ++q3) {
+        const Vec3<Pair<T>> &S = row.S[q3];
+        const Vec3<Pair<T>> nS = neg3(S);
+#pragma unroll
+        for (int q2 = 0; q2 < 2; ++q2) {
+            const Vec3<Pair<T>> R = both3(row.R[q2][q3]);
+            const Vec3<Pair<T>> &U = row.U[q2];
+            const Vec3<Pair<T>> C0 = cross3(S, nS, U), C1 = cross3(U, nU[q2], R);
+            // R x S = -(S x R) = (-S) x R
+            const Vec3<Pair<T>> C2 = cross3(nS, S, R);
+            det[q2][q3] = dot3(R, C0);
+            const Pair<T> inv = neg_rcp_abs(det[q2][q3]);
+            const Pair<T> id = inv * wd, ic = inv * wc;
+            Pair<T>(&m)[6] = M[q2][q3];
+            m[0] = dot3(C0, C0) * id;
+            m[1] = dot3(C1, C1) * id;
+            m[2] = dot3(C2, C2) * id;
+            m[3] = dot3(C0, C1) * ic;
+            m[4] = dot3(C0, C2) * ic;
+            m[5] = dot3(C1, C2) * ic;
+        }
+    }
+}
+
+// T[c][d] = sum_{u,v} A[u][v] 6F_c(u) 6F_d(v); A[v] and the rows c = 0, 1 are pairs
+// over u and c: To[d] = (T[0][d], T[1][d]), T2[d] = T[2][d].
+template <typename T>
+__device__ __forceinline__ void contract_FF(Pair<T> A0, Pair<T> A1, Pair<T> (&To)[3], T (&T2)[3]) {
+    Pair<T> W[3];
+    prod6(A0, A1, W);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        T o0, o1;
+        prod6(pair_lo(W[d]), pair_hi(W[d]), o0, o1, T2[d]);
+        To[d] = pair(o0, o1);
+    }
+}
+
+// Packed lower k_e (36 entries, p = a(a+1)/2 + b) from brick_M's M.  k_ab is a sum
+// of nine contracted terms:
+//   s1 Trr[c2][c3] + s2 Tss[c1][c3] + s3 Ttt[c1][c2]
+//   + the cross terms in (r,s), (r,t), (s,t),
+// c_i the class of the pair's bits on axis i (0, 1, or 2 = mixed) and s_i = -1 for
+// mixed bits.  Pairs of nodes with equal bits on axis 1 come two at a time (bit 0
+// and 1), the 16 with mixed bits one by one; sums that several entries share are
+// formed once.
+template <typename T>
+__device__ __forceinline__ void brick_contract(const Pair<T> (&M)[2][2][6], T (&k)[36]) {
+    // (c1 = 0, 1) as pairs, c1 = 2 as scalars
+    Pair<T> Tss[3], Ttt[3];  // [c3], [c2]
+    T Tss2[3], Ttt2[3], Trr[3][3];
+    {
+        T a[2][2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int v = 0; v < 2; ++v) a[u][v] = pair_lo(M[u][v][0]) + pair_hi(M[u][v][0]);  // sum over q1
+        Pair<T> o[3];
+        T o2[3];
+        contract_FF(pair(a[0][0], a[1][0]), pair(a[0][1], a[1][1]), o, o2);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) Trr[0][d] = pair_lo(o[d]), Trr[1][d] = pair_hi(o[d]), Trr[2][d] = o2[d];
+    }
+    contract_FF(M[0][0][1] + M[1][0][1], M[0][1][1] + M[1][1][1], Tss, Tss2);  // sum over q2
+    contract_FF(M[0][0][2] + M[0][1][2], M[1][0][2] + M[1][1][2], Ttt, Ttt2);  // sum over q3
+    // cross terms: Vrs[x][y][c3], Vrt[x][c2][z] (pairs over x), Vst[c1][y][z]
+    Pair<T> Vrs[2][3], Vrt[3][2], Vst[2][2];
+    T Vst2[2][2];
+    {
+        Pair<T> W[2][3];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) prod6(M[b][0][3], M[b][1][3], W[b]);
+#pragma unroll
+        for (int c3 = 0; c3 < 3; ++c3) {
+            Pair<T> y0, y1;
+            hat_pair(W[0][c3], W[1][c3], y0, y1);
+            Vrs[0][c3] = hat_in_pair(y0);
+            Vrs[1][c3] = hat_in_pair(y1);
+        }
+    }
+    {
+        Pair<T> W[2][2];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) hat_pair(M[b][0][4], M[b][1][4], W[b][0], W[b][1]);
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+            Pair<T> o[3];
+            prod6(W[0][z], W[1][z], o);
+#pragma unroll
+            for (int c2 = 0; c2 < 3; ++c2) Vrt[c2][z] = hat_in_pair(o[c2]);
+        }
+    }
+    {
+        Pair<T> W[2][2];
+#pragma unroll
+        for (int b = 0; b < 2; ++b) hat_pair(M[b][0][5], M[b][1][5], W[b][0], W[b][1]);
+#pragma unroll
+        for (int z = 0; z < 2; ++z) {
+            Pair<T> y[2];
+            hat_pair(W[0][z], W[1][z], y[0], y[1]);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                T o0, o1;
+                prod6(pair_lo(y[b]), pair_hi(y[b]), o0, o1, Vst2[b][z]);
+                Vst[b][z] = pair(o0, o1);
+            }
+        }
+    }
+    // pairs with equal bits on axis 1 (value x): the (r,s) term is
+    // sig(x) (sig(b2) V[x][a2][c3] + sig(a2) V[x][b2][c3]) = sig(x) times 2 sig(a2) V[a2]
+    // for equal bits on axis 2 and V[0] - V[1] for mixed ones; the (r,t) term alike
+    const Pair<T> sig = pair(T(-1), T(1)), sig2 = pair(T(-2), T(2)), msig2 = pair(T(2), T(-2));
+    const Pair<T> two = pair(T(2), T(2)), mtwo = pair(T(-2), T(-2));
+    Pair<T> base[3][3];  // [c2][c3]: all but the (s,t) term
+#pragma unroll
+    for (int c2 = 0; c2 < 3; ++c2)
+#pragma unroll
+        for (int c3 = 0; c3 < 3; ++c3) {
+            Pair<T> v = pair(Trr[c2][c3], Trr[c2][c3]);
+            v = c2 == 2 ? v - Tss[c3] : v + Tss[c3];
+            v = c3 == 2 ? v - Ttt[c2] : v + Ttt[c2];
+            v = c2 == 2 ? pfma(sig, Vrs[0][c3] - Vrs[1][c3], v) : pfma(c2 ? sig2 : msig2, Vrs[c2][c3], v);
+            v = c3 == 2 ? pfma(sig, Vrt[c2][0] - Vrt[c2][1], v) : pfma(c3 ? sig2 : msig2, Vrt[c2][c3], v);
+            base[c2][c3] = v;
+        }
+    auto put = [&](int a, int b, T v) { k[a > b ? a * (a + 1) / 2 + b : b * (b + 1) / 2 + a] = v; };
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q <= p; ++q) {
+            const int a2 = p >> 1, a3 = p & 1, b2 = q >> 1, b3 = q & 1;
+            const int c2 = hcls(a2, b2), c3 = hcls(a3, b3);
+            Pair<T> v = base[c2][c3];
+            if (c2 != 2 && c3 != 2) v = pfma(a2 == a3 ? two : mtwo, Vst[a2][a3], v);
+            else if (c3 != 2) v = a3 ? v + (Vst[0][a3] - Vst[1][a3]) : v - (Vst[0][a3] - Vst[1][a3]);
+            else if (c2 != 2) v = a2 ? v + (Vst[a2][0] - Vst[a2][1]) : v - (Vst[a2][0] - Vst[a2][1]);
+            else if (a2 == a3) v = v - (Vst[0][1] + Vst[1][0]);
+            else v = v + (Vst[0][0] + Vst[1][1]);
+            put(hnode(0, a2, a3), hnode(0, b2, b3), pair_lo(v));
+            put(hnode(1, a2, a3), hnode(1, b2, b3), pair_hi(v));
+        }
+    // pairs with mixed bits on axis 1: node (1, a2, a3) against (0, b2, b3)
+    T rs[2][2][3], rt[3][2][2], st[4][4], base2[3][3];
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                // sig(b2) V[0][a2] - sig(a2) V[1][b2], (x, y) = (a2, b2); alike in (r,t)
+                const T u = pair_lo(Vrs[x][c]), w = pair_hi(Vrs[y][c]);
+                rs[x][y][c] = y ? (x ? u - w : u + w) : (x ? -u - w : w - u);
+                const T ut = pair_lo(Vrt[c][x]), wt = pair_hi(Vrt[c][y]);
+                rt[c][x][y] = y ? (x ? ut - wt : ut + wt) : (x ? -ut - wt : wt - ut);
+            }
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q <= p; ++q) {
+            const int a2 = p >> 1, a3 = p & 1, b2 = q >> 1, b3 = q & 1;
+            const T u = Vst2[b2][a3], w = Vst2[a2][b3];
+            // sig(a2) sig(b3) V[b2][a3] + sig(a3) sig(b2) V[a2][b3]
+            st[p][q] = st[q][p] = (a2 == b3 ? u : -u) + (a3 == b2 ? w : -w);
+        }
+#pragma unroll
+    for (int c2 = 0; c2 < 3; ++c2)
+#pragma unroll
+        for (int c3 = 0; c3 < 3; ++c3)
+            base2[c2][c3] = (c2 == 2 ? -Tss2[c3] : Tss2[c3]) + (c3 == 2 ? -Ttt2[c2] : Ttt2[c2]) - Trr[c2][c3];
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int a2 = p >> 1, a3 = p & 1, b2 = q >> 1, b3 = q & 1;
+            const int c2 = hcls(a2, b2), c3 = hcls(a3, b3);
+            put(hnode(1, a2, a3), hnode(0, b2, b3), base2[c2][c3] + rs[a2][b2][c3] + rt[c2][a3][b3] + st[p][q]);
+        }
 }
 
 // Full brick element: packed k_e in precision T from node coordinates in S.
 template <typename T, typename S>
 __device__ __forceinline__ void brick_ke(const S (*xc)[3], T c, T (&k)[36]) {
-    Vec3<T> e[3][2][2];
-    brick_edges<T, S>(xc, e);
-    Vec3<T> row[3][2][2];
-    brick_jrows(e, row);
-    T M[8][6], det[8];
+    BrickRows<T> row;
+    brick_rows<T, S>(xc, row);
+    Pair<T> M[2][2][6], det[2][2];
     brick_M(row, c * T(0.125), M, det);
     brick_contract(M, k);
+}
+
+// Whether an element is distorted: max_q det J > thr min_q det J, or a det J <= 0.
+template <typename T>
+__device__ __forceinline__ bool brick_distorted(const Pair<T> (&det)[2][2], float thr) {
+    T lo = pair_lo(det[0][0]), hi = lo;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const T a = pair_lo(det[q >> 1][q & 1]), b = pair_hi(det[q >> 1][q & 1]);
+        lo = fmin(lo, fmin(a, b));
+        hi = fmax(hi, fmax(a, b));
+    }
+    return !(lo > T(0)) || hi > T(thr) * lo;
+}
+
+// The FP64 M_q of a distorted element, rounded to floats: Ml[24][2] in the order of
+// brick_M's pairs.  A call, not inlined: a few elements in a million take it, and
+// inlined its registers would spill the FP32 path's.
+template <typename S>
+__device__ __noinline__ void brick_M_distorted(const S (*xc)[3], float c, float (*Ml)[2]) {
+    BrickRows<double> row;
+    brick_rows<double, S>(xc, row);
+    Pair<double> M[2][2][6], det[2][2];
+    brick_M(row, (double)c * 0.125, M, det);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+            Ml[6 * q + i][0] = (float)M[q >> 1][q & 1][i].x;
+            Ml[6 * q + i][1] = (float)M[q >> 1][q & 1][i].y;
+        }
 }
 
 // Mixed precision brick: FP32 throughout, except that an element whose ratio
@@ -371,30 +639,23 @@ __device__ __forceinline__ void brick_ke(const S (*xc)[3], T c, T (&k)[36]) {
 // Returns true when the FP64 path was taken.
 template <typename S>
 __device__ __forceinline__ bool brick_ke_mixed(const S (*xc)[3], float c, float thr, float (&k)[36]) {
-    Vec3<float> e[3][2][2];
-    brick_edges<float, S>(xc, e);
-    Vec3<float> row[3][2][2];
-    brick_jrows(e, row);
-    float M[8][6], det[8];
+    BrickRows<float> row;
+    brick_rows<float, S>(xc, row);
+    Pair<float> M[2][2][6], det[2][2];
     brick_M(row, c * 0.125f, M, det);
-    float dmin = det[0], dmax = det[0];
-#pragma unroll
-    for (int q = 1; q < 8; ++q) {
-        dmin = fminf(dmin, det[q]);
-        dmax = fmaxf(dmax, det[q]);
-    }
-    const bool flagged = !(dmin > 0.f) || dmax > thr * dmin;
+    const bool flagged = brick_distorted(det, thr);
     if (flagged) {
-        Vec3<double> ed[3][2][2];
-        brick_edges<double, S>(xc, ed);
-        Vec3<double> rowd[3][2][2];
-        brick_jrows(ed, rowd);
-        double Md[8][6], detd[8];
-        brick_M(rowd, (double)c * 0.125, Md, detd);
+        S xl[8][3];  // copies: only these live in local memory
+        float Ml[24][2];
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
+        for (int a = 0; a < 8; ++a)
 #pragma unroll
-            for (int i = 0; i < 6; ++i) M[q][i] = (float)Md[q][i];
+            for (int d = 0; d < 3; ++d) xl[a][d] = xc[a][d];
+        brick_M_distorted<S>(xl, c, Ml);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int i = 0; i < 6; ++i) M[q >> 1][q & 1][i] = pair(Ml[6 * q + i][0], Ml[6 * q + i][1]);
     }
     brick_contract(M, k);
     return flagged;
