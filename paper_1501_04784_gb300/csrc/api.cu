@@ -221,6 +221,9 @@ fem_status fem_mesh_create(fem_mesh *out, fem_elem type, int64_t n_nodes, int64_
         return FEM_ERR_ARG;
     }
     m->arena.budget = m->opt.mem_budget_bytes;
+    // slabs of about the size of a mesh's larger plan arrays: 64 MB from 1M bricks on,
+    // 256 KB for a few thousand elements
+    m->arena.slab = std::min<size_t>((size_t)64 << 20, std::max<size_t>((size_t)256 << 10, (size_t)n_elems * m->npe * 8));
     cudaStream_t s = as_stream(stream);
     fem_status st = m->status.alloc(m->arena, 1, "status word");
     {
@@ -248,6 +251,7 @@ void fem_mesh_destroy(fem_mesh m) {
     if (!m) return;
     cudaDeviceSynchronize();
     batch_forget(m);
+    m->arena.closing = true;
     delete m;
 }
 

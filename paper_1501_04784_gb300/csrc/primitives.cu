@@ -2,6 +2,7 @@
 // scan and radix sort used by the symbolic phase.
 #include <cstdarg>
 #include <cstring>
+#include <iterator>
 
 #include "common.cuh"
 
@@ -33,7 +34,18 @@ int64_t launch_count(int reset) {
 
 fem_status Arena::alloc(void **p, size_t bytes, const char *what) {
     *p = nullptr;
-    const size_t need = bytes ? bytes : 1;
+    size_t need = bytes ? bytes : 1;
+    if (!budget && slab && need <= slab / 2) {
+        need = (need + 255) & ~(size_t)255;
+        *p = carve(need);
+        if (*p) {
+            live += need;
+            block[*p] = need;
+            if (live > peak) peak = live;
+            return FEM_OK;
+        }
+        cudaGetLastError();  // no room for a slab: a block of its own
+    }
     // a kept block of at least the size and at most twice it (the smallest such)
     size_t best = pool.size();
     for (size_t i = 0; i < pool.size(); ++i)
@@ -80,6 +92,12 @@ void Arena::release(void *p, size_t bytes) {
     const size_t sz = it != block.end() ? it->second : bytes;
     if (it != block.end()) block.erase(it);
     live -= sz;
+    // a range may be handed out again at once: outside a symbolic phase (one stream)
+    // the device is waited for, as cudaFree does
+    if (!slabs.empty()) {
+        if (!keep && !closing) cudaDeviceSynchronize();
+        if (uncarve(p, sz)) return;
+    }
     if (keep) {
         pool.emplace_back(p, sz);
         kept += sz;
@@ -92,6 +110,66 @@ void Arena::trim() {
     for (auto &b : pool) cudaFree(b.first);
     pool.clear();
     kept = 0;
+    for (size_t i = 0; i < slabs.size();) {
+        Slab &s = slabs[i];
+        if (s.holes.size() == 1 && s.holes.begin()->second == s.size) {
+            cudaFree(s.base);
+            slabs.erase(slabs.begin() + (std::ptrdiff_t)i);
+        } else {
+            ++i;
+        }
+    }
+}
+
+Arena::~Arena() {
+    trim();
+    for (Slab &s : slabs) cudaFree(s.base);
+}
+
+// The smallest free range of the slabs that holds `need` bytes, or a new slab's start;
+// null if no slab can be had.
+void *Arena::carve(size_t need) {
+    Slab *best = nullptr;
+    std::map<size_t, size_t>::iterator hole;
+    for (Slab &s : slabs)
+        for (auto it = s.holes.begin(); it != s.holes.end(); ++it)
+            if (it->second >= need && (!best || it->second < hole->second)) best = &s, hole = it;
+    if (!best) {
+        void *base = nullptr;
+        if (cudaMalloc(&base, slab) != cudaSuccess) return nullptr;
+        slabs.push_back(Slab{static_cast<char *>(base), slab, {{0, slab}}});
+        best = &slabs.back();
+        hole = best->holes.begin();
+    }
+    const size_t off = hole->first, len = hole->second;
+    best->holes.erase(hole);
+    if (len > need) best->holes[off + need] = len - need;
+    return best->base + off;
+}
+
+// Returns a range to its slab (joined with the free ranges beside it); false if p is
+// not in a slab.
+bool Arena::uncarve(void *p, size_t size) {
+    char *c = static_cast<char *>(p);
+    for (Slab &s : slabs) {
+        if (c < s.base || c >= s.base + s.size) continue;
+        size_t off = (size_t)(c - s.base), len = size;
+        auto next = s.holes.lower_bound(off);
+        if (next != s.holes.end() && next->first == off + len) {
+            len += next->second;
+            next = s.holes.erase(next);
+        }
+        if (next != s.holes.begin()) {
+            auto prev = std::prev(next);
+            if (prev->first + prev->second == off) {
+                prev->second += len;
+                return true;
+            }
+        }
+        s.holes[off] = len;
+        return true;
+    }
+    return false;
 }
 
 int num_sms() {
