@@ -354,8 +354,11 @@ static PatchArgs patch_args(fem_mesh m, fem_prec p, bool fused) {
     a.threads = m->opt.block_threads > 0 ? m->opt.block_threads : 256;
     if (a.threads > patch_max_threads(m->npe)) a.threads = patch_max_threads(m->npe);
     a.threads = (a.threads + 31) / 32 * 32;
+    // assembling given element matrices, one block fills an SM's shared memory
+    if (!fused && m->opt.block_threads <= 0 && m->plan.full.lists.ready) a.threads = 512;
     if (is_elastic(m)) a.threads = elastic_threads(m->npe, m->opt.block_threads);  // its own default and cap
     a.blocks_per_sm = m->opt.blocks_per_sm;
+    if (fused && a.mixed && m->xrank.n >= 4 * (size_t)m->n_nodes) a.xrank = m->xrank.ptr;
     a.mode = kernel_mode(m->opt);
     a.wait = wait_ctl(m);
     return a;
@@ -585,6 +588,7 @@ static fem_status chunk_pipeline(fem_mesh m, fem_prec p, const void *X, fem_dtyp
             a.closure = &cl;
             return launch_patch(a, s);
         }));
+        a.x_ordered = true;
         FEM_CUDA(cudaEventRecord(m->chunk_built[j], s));
         FEM_CUDA(cudaStreamWaitEvent(m->copy_stream, m->chunk_built[j], 0));
         FEM_CUDA(cudaMemcpyAsync(host + v0 * w, dst, nv * w, cudaMemcpyDeviceToHost, m->copy_stream));

@@ -27,6 +27,8 @@ struct BatchCtx {
     int npe = 8;
     bool elastic = false;  // the elasticity operator (operator_kind 2)
     bool tiles = false;    // the meshes build on element tiles
+    bool gather = false;   // every mesh has gather lists
+    GatherPatch *d_gpatch = nullptr;
     BatchItem *d_items = nullptr;
     TileBatchItem *d_titems = nullptr;
     std::vector<TileBatchItem> h_titems;
@@ -42,6 +44,7 @@ struct BatchCtx {
         if (exec) cudaGraphExecDestroy(exec);
         if (graph) cudaGraphDestroy(graph);
         if (d_items) cudaFree(d_items);
+        if (d_gpatch) cudaFree(d_gpatch);
         if (d_titems) cudaFree(d_titems);
         if (d_prefix) cudaFree(d_prefix);
         if (d_bprefix) cudaFree(d_bprefix);
@@ -77,7 +80,8 @@ static void fill_items(BatchCtx &c, const void *const *X, const void *const *cc,
         return;
     }
     for (size_t i = 0; i < c.meshes.size(); ++i) {
-        c.h_items[i] = BatchItem{c.meshes[i]->plan.view(), X[i], cc[i], vals[i], mesh_threshold(c.meshes[i]), 0};
+        c.h_items[i] = BatchItem{c.meshes[i]->plan.view(), X[i], cc[i], vals[i],
+                                 mesh_threshold(c.meshes[i]), 0};
         // the elasticity operator's values: the DOF matrix (bounds of the debug build)
         if (c.elastic) c.h_items[i].pv.nnz = 9 * c.meshes[i]->nnz - 3 * c.meshes[i]->n_nodes;
     }
@@ -101,6 +105,7 @@ static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *cons
     std::vector<int64_t> prefix(n + 1, 0), bprefix(n + 1, 0);
     PlanMax pm;
     TileMax tm;
+    GatherMax gm;
     for (int i = 0; i < n; ++i) {
         if (c.tiles) {
             prefix[i + 1] = prefix[i] + c.meshes[i]->tiles.n_tiles;
@@ -109,6 +114,7 @@ static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *cons
         } else {
             prefix[i + 1] = prefix[i] + c.meshes[i]->plan.n_patches;
             pm.add(c.meshes[i]->plan);
+            gm.add(c.meshes[i]->plan);
         }
     }
     if (c.tiles) FEM_CUDA(cudaMalloc(&c.d_titems, n * sizeof(TileBatchItem)));
@@ -118,6 +124,12 @@ static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *cons
     if (c.tiles) {
         FEM_CUDA(cudaMalloc(&c.d_bprefix, (n + 1) * sizeof(int64_t)));
         FEM_CUDA(cudaMemcpyAsync(c.d_bprefix, bprefix.data(), (n + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    }
+    if (c.gather) {
+        FEM_CUDA(cudaMalloc(&c.d_gpatch, std::max<int64_t>(prefix[n], 1) * sizeof(GatherPatch)));
+        for (int i = 0; i < n; ++i)
+            FEM_TRY(launch_gather_table(c.meshes[i]->plan.full.lists.patch.ptr, prefix[i + 1] - prefix[i], i,
+                                        c.d_gpatch + prefix[i], s));
     }
     c.h_items.resize(n);
     c.h_titems.resize(n);
@@ -153,11 +165,14 @@ static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *cons
         bl.titems = c.d_titems;
         bl.bprefix = c.d_bprefix;
         bl.prefix = c.d_prefix;
+        bl.gpatch = c.d_gpatch;
+        bl.n_work = prefix[n];
         bl.n = n;
         bl.mode = kernel_mode(c.meshes[0]->opt);
         bl.wait = wait_ctl(c.meshes[0]);
         const fem_status cs = c.elastic ? elastic_batched_config(c.npe, c.mixed, pm, cd.first, cd.second, &bl)
                               : c.tiles ? tile_batched_config(c.npe, c.mixed, tm, cd.first, cd.second, &bl)
+                              : c.gather ? gather_batched_config(c.npe, c.mixed, gm, cd.first, cd.second, &bl)
                                         : batched_config(c.npe, c.mixed, pm, cd.first, cd.second, &bl);
         if (cs != FEM_OK) continue;
         FEM_TRY(launch_batched_kernel(bl, s));  // warm-up
@@ -232,6 +247,18 @@ fem_status launch_batched(const fem_mesh *ms, int n, bool mixed, bool tiles, con
         set_error("batched builds take %s X and c", mixed ? "float" : "double");
         return FEM_ERR_UNSUPPORTED;
     }
+    // gather lists when every mesh of the batch has them, else the scatter for all
+    // (a mesh planned for it anew leaves the batch cache, so this comes first)
+    bool gather = !tiles && !elastic;
+    for (int i = 0; i < n; ++i) gather = gather && ms[i]->plan.full.lists.ready;
+    if (!gather && !tiles && !elastic)
+        for (int i = 0; i < n; ++i) {
+            FEM_TRY(ensure_targets(ms[i], s));
+            if (ms[i]->plan.chunked) {
+                set_error("mesh %d of the batch is planned in groups under its memory budget", i);
+                return FEM_ERR_UNSUPPORTED;
+            }
+        }
     std::lock_guard<std::mutex> lock(g_batch_mu);
     BatchCtx *ctx = find_ctx(ms, n, mixed, tiles, xd, cd);
     if (!ctx) {
@@ -243,6 +270,7 @@ fem_status launch_batched(const fem_mesh *ms, int n, bool mixed, bool tiles, con
         nc->cd = cd;
         nc->npe = npe;
         nc->elastic = elastic;
+        nc->gather = gather;
         FEM_TRY(create_ctx(*nc, X, c, vals, s));
         if (g_batch_ctx.size() >= MAX_BATCH_CTX) g_batch_ctx.erase(g_batch_ctx.begin());
         g_batch_ctx.push_back(std::move(nc));

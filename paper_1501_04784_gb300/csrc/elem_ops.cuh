@@ -59,6 +59,20 @@ __device__ __forceinline__ bool element_matrix(const S (*xc)[3], CT ce, float th
     }
 }
 
+// The same, except that a distorted brick in mixed precision is left for later: it
+// returns true, and brick_distorted_shared gives its matrix.
+template <int NPE, typename AccT, typename S, bool MIXED, typename CT>
+__device__ __forceinline__ bool element_matrix_fast(const S (*xc)[3], CT ce, float thr, unsigned mode,
+                                                    AccT (&k)[ElemTraits<NPE>::NP]) {
+    if constexpr (MIXED && NPE == 8) {
+        return (mode & OP_MASS) ? brick_me_fp32<S>(xc, static_cast<float>(ce), thr, k)
+                                : brick_ke_fp32<S>(xc, static_cast<float>(ce), thr, k);
+    } else {
+        element_matrix<NPE, AccT, S, MIXED>(xc, ce, thr, mode, k);
+        return false;
+    }
+}
+
 // Knuth's TwoSum: s + err == a + b exactly (round-to-nearest, no reassociation).
 __device__ __forceinline__ void two_sum_acc(float2 &acc, float x) {
     const float s = acc.x + x;

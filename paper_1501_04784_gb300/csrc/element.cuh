@@ -202,57 +202,6 @@ __device__ __forceinline__ void brick_jrows(const Vec3<T> (&e)[3][2][2], Vec3<T>
     }
 }
 
-// Contract one Gauss axis of m[8] (index 4 q1 + 2 q2 + q3) with the hats
-// (kind 0: phi_x, 2 outputs) or the hat products (kind 1: F_c, 3 outputs).
-// The cross terms need V[x or c][y or c][z or c] over the three axes in turn.
-template <typename T, int K1, int K2, int K3>
-__device__ __forceinline__ void contract_cross(const T (&m)[2][2][2], T (&V)[3][3][3]) {
-    const T PP = T(FEM_GPP), QQ = T(FEM_GQQ), PQ = T(FEM_GPQ);
-    constexpr int N1 = K1 ? 3 : 2, N2 = K2 ? 3 : 2, N3 = K3 ? 3 : 2;
-    T W[2][2][3];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const T m0 = m[a][b][0], m1 = m[a][b][1];
-            if (K3) {
-                W[a][b][0] = PP * m0 + QQ * m1;
-                W[a][b][1] = QQ * m0 + PP * m1;
-                W[a][b][2] = PQ * (m0 + m1);
-            } else {
-                hat_pair(m0, m1, W[a][b][0], W[a][b][1]);
-            }
-        }
-    T Y[2][3][3];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int k = 0; k < N3; ++k) {
-            const T w0 = W[a][0][k], w1 = W[a][1][k];
-            if (K2) {
-                Y[a][0][k] = PP * w0 + QQ * w1;
-                Y[a][1][k] = QQ * w0 + PP * w1;
-                Y[a][2][k] = PQ * (w0 + w1);
-            } else {
-                hat_pair(w0, w1, Y[a][0][k], Y[a][1][k]);
-            }
-        }
-#pragma unroll
-    for (int j = 0; j < N2; ++j)
-#pragma unroll
-        for (int k = 0; k < N3; ++k) {
-            const T y0 = Y[0][j][k], y1 = Y[1][j][k];
-            if (K1) {
-                V[0][j][k] = PP * y0 + QQ * y1;
-                V[1][j][k] = QQ * y0 + PP * y1;
-                V[2][j][k] = PQ * (y0 + y1);
-            } else {
-                hat_pair(y0, y1, V[0][j][k], V[1][j][k]);
-            }
-        }
-    (void)N1;
-}
-
 // ------------------------------------------------------ brick stiffness, in pairs
 // The brick's arithmetic runs on pairs (pair.cuh): every quantity that depends on
 // the Gauss point index q1 is held for q1 = 0 and 1 together, so FP32 needs one
@@ -615,28 +564,95 @@ __device__ __forceinline__ bool brick_distorted(const Pair<T> (&det)[2][2], floa
     return !(lo > T(0)) || hi > T(thr) * lo;
 }
 
-// The FP64 M_q of a distorted element, rounded to floats: Ml[24][2] in the order of
-// brick_M's pairs.  A call, not inlined: a few elements in a million take it, and
-// inlined its registers would spill the FP32 path's.
+// Distorted bricks (mixed precision): a brick whose max_q det J / min_q det J exceeds
+// the threshold (or with a det J <= 0) takes its M_q, or determinants, from FP64.
+
+// Gauss point q = 4 q1 + 2 q2 + q3 of a brick in FP64 from its node coordinates (edge
+// differences formed in S): M[0..5] as brick_M scales it (s = c / 8), rounded to
+// floats; M[6] = det 2J_q.  One copy of the code, so that every kernel gets the same
+// bits; a few elements in a million come here.
 template <typename S>
-__device__ __noinline__ void brick_M_distorted(const S (*xc)[3], float c, float (*Ml)[2]) {
-    BrickRows<double> row;
-    brick_rows<double, S>(xc, row);
-    Pair<double> M[2][2][6], det[2][2];
-    brick_M(row, (double)c * 0.125, M, det);
+__device__ __noinline__ void brick_point(const S (*x)[3], int q, double s, float *M) {
+    const int g[3] = {q >> 2, (q >> 1) & 1, q & 1};
+    double w[3][2];  // the hats of each axis at the point
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        w[ax][0] = g[ax] ? FEM_GQ : FEM_GP;
+        w[ax][1] = g[ax] ? FEM_GP : FEM_GQ;
+    }
+    double row[3][3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int ax = 0; ax < 3; ++ax) {
+            double v = 0.0;
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const int n0 = ax == 0 ? hnode(0, i, j) : ax == 1 ? hnode(i, 0, j) : hnode(i, j, 0);
+                    const int n1 = ax == 0 ? hnode(1, i, j) : ax == 1 ? hnode(i, 1, j) : hnode(i, j, 1);
+                    v = fma(w[ax == 0 ? 1 : 0][i] * w[ax == 2 ? 1 : 2][j], (double)(x[n1][d] - x[n0][d]), v);
+                }
+            row[ax][d] = v;
+        }
+    const Vec3<double> R = {row[0][0], row[0][1], row[0][2]}, Sv = {row[1][0], row[1][1], row[1][2]},
+                       U = {row[2][0], row[2][1], row[2][2]};
+    const Vec3<double> C0 = cross3(Sv, U), C1 = cross3(U, R), C2 = cross3(R, Sv);
+    const double d = dot3(R, C0), inv = rcp_rn(fabs(d)) * s;
+    M[0] = (float)(dot3(C0, C0) * inv * (1.0 / 36.0));
+    M[1] = (float)(dot3(C1, C1) * inv * (1.0 / 36.0));
+    M[2] = (float)(dot3(C2, C2) * inv * (1.0 / 36.0));
+    M[3] = (float)(dot3(C0, C1) * inv * (1.0 / 6.0));
+    M[4] = (float)(dot3(C0, C2) * inv * (1.0 / 6.0));
+    M[5] = (float)(dot3(C1, C2) * inv * (1.0 / 6.0));
+    M[6] = (float)d;
+}
+
+// All eight points by the calling lane.
+template <typename S>
+__device__ __noinline__ void brick_points(const S (*x)[3], float c, float (*M)[7]) {
+    for (int q = 0; q < 8; ++q) brick_point<S>(x, q, (double)c * 0.125, M[q]);
+}
+
+// All eight points of one element by eight consecutive lanes (q = lane & 7), the
+// results to all of them.  One lane alone runs some 900 FP64 instructions of about 60
+// cycles each, 20 us, for which its whole block waits at the next barrier: the one such
+// block among a few hundred decided the kernel's time.
+template <typename S>
+__device__ __forceinline__ void brick_points_shared(const S (*x)[3], float c, float (&M)[8][7]) {
+    float m[7];
+    brick_point<S>(x, threadIdx.x & 7, (double)c * 0.125, m);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int i = 0; i < 7; ++i) M[q][i] = __shfl_sync(0xffffffffu, m[i], q, 8);
+}
+
+__device__ __forceinline__ void pairs_of_points(const float (&P)[8][7], Pair<float> (&M)[2][2][6]) {
 #pragma unroll
     for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            Ml[6 * q + i][0] = (float)M[q >> 1][q & 1][i].x;
-            Ml[6 * q + i][1] = (float)M[q >> 1][q & 1][i].y;
-        }
+        for (int i = 0; i < 6; ++i) M[q >> 1][q & 1][i] = pair(P[q][i], P[4 + q][i]);
+}
+__device__ __forceinline__ void pairs_of_dets(const float (&P)[8][7], Pair<float> (&det)[2][2]) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) det[q >> 1][q & 1] = pair(P[q][6], P[4 + q][6]);
 }
 
-// Mixed precision brick: FP32 throughout, except that an element whose ratio
-// max_q det J / min_q det J exceeds `thr` (or with a det J <= 0) recomputes its
-// Jacobians, determinants and M_q in FP64 from the coordinate differences.
-// Returns true when the FP64 path was taken.
+// Brick in FP32; returns whether it is distorted (then k is not its final matrix).
+template <typename S>
+__device__ __forceinline__ bool brick_ke_fp32(const S (*xc)[3], float c, float thr, float (&k)[36]) {
+    BrickRows<float> row;
+    brick_rows<float, S>(xc, row);
+    Pair<float> M[2][2][6], det[2][2];
+    brick_M(row, c * 0.125f, M, det);
+    brick_contract(M, k);
+    return brick_distorted(det, thr);
+}
+
+// Mixed precision brick: FP32 throughout, except for the FP64 M_q of a distorted
+// element.  Returns true when the FP64 path was taken.
 template <typename S>
 __device__ __forceinline__ bool brick_ke_mixed(const S (*xc)[3], float c, float thr, float (&k)[36]) {
     BrickRows<float> row;
@@ -645,17 +661,14 @@ __device__ __forceinline__ bool brick_ke_mixed(const S (*xc)[3], float c, float 
     brick_M(row, c * 0.125f, M, det);
     const bool flagged = brick_distorted(det, thr);
     if (flagged) {
-        S xl[8][3];  // copies: only these live in local memory
-        float Ml[24][2];
+        S x[8][3];  // copies: only these live in local memory
+        float P[8][7];
 #pragma unroll
         for (int a = 0; a < 8; ++a)
 #pragma unroll
-            for (int d = 0; d < 3; ++d) xl[a][d] = xc[a][d];
-        brick_M_distorted<S>(xl, c, Ml);
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-            for (int i = 0; i < 6; ++i) M[q >> 1][q & 1][i] = pair(Ml[6 * q + i][0], Ml[6 * q + i][1]);
+            for (int d = 0; d < 3; ++d) x[a][d] = xc[a][d];
+        brick_points<S>(x, c, P);
+        pairs_of_points(P, M);
     }
     brick_contract(M, k);
     return flagged;
@@ -668,69 +681,84 @@ __device__ __forceinline__ bool brick_ke_mixed(const S (*xc)[3], float c, float 
 // D[q1][q2][q3] = |det J_q| and V = D contracted with the hat products F_c on every
 // axis, M_ab = c V[cls(a1,b1)][cls(a2,b2)][cls(a3,b3)].  det(2 J_q) = 8 det J_q.
 template <typename T>
-__device__ __forceinline__ void brick_dets(const Vec3<T> (&row)[3][2][2], T (&det)[8]) {
+__device__ __forceinline__ void brick_dets(const BrickRows<T> &row, Pair<T> (&det)[2][2]) {
 #pragma unroll
-    for (int q1 = 0; q1 < 2; ++q1)
+    for (int q3 = 0; q3 < 2; ++q3) {
+        const Vec3<Pair<T>> nS = neg3(row.S[q3]);
 #pragma unroll
         for (int q2 = 0; q2 < 2; ++q2)
-#pragma unroll
-            for (int q3 = 0; q3 < 2; ++q3)
-                det[4 * q1 + 2 * q2 + q3] = dot3(row[0][q2][q3], cross3(row[1][q1][q3], row[2][q1][q2]));
+            det[q2][q3] = dot3(both3(row.R[q2][q3]), cross3(row.S[q3], nS, row.U[q2]));
+    }
 }
 
 template <typename T>
-__device__ __forceinline__ void brick_mass_from_dets(const T (&det)[8], T c, T (&m)[36]) {
-    T D[2][2][2];
+__device__ __forceinline__ Pair<T> pair_abs(Pair<T> p) {
+    const T a = pair_lo(p), b = pair_hi(p);
+    return pair(a < T(0) ? -a : a, b < T(0) ? -b : b);
+}
+
+// Packed mass matrix from det(2 J_q): the determinants contracted with the hat
+// products (times 6, see prod6) on every axis, as pairs over the classes 0 and 1 of
+// axis 1.
+template <typename T>
+__device__ __forceinline__ void brick_mass_from_dets(const Pair<T> (&det)[2][2], T c, T (&m)[36]) {
+    Pair<T> W[2][3], Y[3][3];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) D[q >> 2][(q >> 1) & 1][q & 1] = det[q] < T(0) ? -det[q] : det[q];
+    for (int q2 = 0; q2 < 2; ++q2) prod6(pair_abs(det[q2][0]), pair_abs(det[q2][1]), W[q2]);
+#pragma unroll
+    for (int c3 = 0; c3 < 3; ++c3) {
+        Pair<T> o[3];
+        prod6(W[0][c3], W[1][c3], o);
+#pragma unroll
+        for (int c2 = 0; c2 < 3; ++c2) Y[c2][c3] = o[c2];
+    }
+    const T s = c * T(0.125 / 216.0);
     T V[3][3][3];
-    contract_cross<T, 1, 1, 1>(D, V);
-    const T s = c * T(0.125);
+#pragma unroll
+    for (int c2 = 0; c2 < 3; ++c2)
+#pragma unroll
+        for (int c3 = 0; c3 < 3; ++c3) {
+            T o0, o1, o2;
+            prod6(pair_lo(Y[c2][c3]), pair_hi(Y[c2][c3]), o0, o1, o2);
+            V[0][c2][c3] = s * o0, V[1][c2][c3] = s * o1, V[2][c2][c3] = s * o2;
+        }
 #pragma unroll
     for (int a = 0; a < 8; ++a)
 #pragma unroll
         for (int b = 0; b <= a; ++b)
-            m[a * (a + 1) / 2 + b] = s * V[hcls(hb1(a), hb1(b))][hcls(hb2(a), hb2(b))][hcls(hb3(a), hb3(b))];
+            m[a * (a + 1) / 2 + b] = V[hcls(hb1(a), hb1(b))][hcls(hb2(a), hb2(b))][hcls(hb3(a), hb3(b))];
 }
 
 template <typename T, typename S>
 __device__ __forceinline__ void brick_me(const S (*xc)[3], T c, T (&m)[36]) {
-    Vec3<T> e[3][2][2];
-    brick_edges<T, S>(xc, e);
-    Vec3<T> row[3][2][2];
-    brick_jrows(e, row);
-    T det[8];
+    BrickRows<T> row;
+    brick_rows<T, S>(xc, row);
+    Pair<T> det[2][2];
     brick_dets(row, det);
     brick_mass_from_dets(det, c, m);
 }
 
-// Brick determinants |det(2 J_q)| at the 8 Gauss points in precision T; with
+// Brick determinants det(2 J_q) at the 8 Gauss points in precision T; with
 // `mixed`, FP32 unless max_q det J / min_q det J exceeds thr (or some det J <= 0),
 // then from FP64.  Returns true when FP64 was used.
 template <typename T, typename S>
-__device__ __forceinline__ bool brick_gauss_dets(const S (*xc)[3], float thr, bool mixed, T (&det)[8]) {
-    Vec3<T> e[3][2][2];
-    brick_edges<T, S>(xc, e);
-    Vec3<T> row[3][2][2];
-    brick_jrows(e, row);
+__device__ __forceinline__ bool brick_gauss_dets(const S (*xc)[3], float thr, bool mixed, Pair<T> (&det)[2][2]) {
+    BrickRows<T> row;
+    brick_rows<T, S>(xc, row);
     brick_dets(row, det);
-    if (!mixed) return false;
-    T dmin = det[0], dmax = det[0];
+    bool flagged = false;
+    if constexpr (sizeof(T) == 4) {
+        flagged = mixed && brick_distorted(det, thr);
+        if (flagged) {
+            S x[8][3];
+            float P[8][7];
 #pragma unroll
-    for (int q = 1; q < 8; ++q) {
-        dmin = det[q] < dmin ? det[q] : dmin;
-        dmax = det[q] > dmax ? det[q] : dmax;
-    }
-    const bool flagged = !(dmin > T(0)) || dmax > T(thr) * dmin;
-    if (flagged) {
-        Vec3<double> ed[3][2][2];
-        brick_edges<double, S>(xc, ed);
-        Vec3<double> rowd[3][2][2];
-        brick_jrows(ed, rowd);
-        double detd[8];
-        brick_dets(rowd, detd);
+            for (int a = 0; a < 8; ++a)
 #pragma unroll
-        for (int q = 0; q < 8; ++q) det[q] = (T)detd[q];
+                for (int d = 0; d < 3; ++d) x[a][d] = xc[a][d];
+            brick_points<S>(x, 0.f, P);
+            pairs_of_dets(P, det);
+        }
     }
     return flagged;
 }
@@ -738,45 +766,56 @@ __device__ __forceinline__ bool brick_gauss_dets(const S (*xc)[3], float thr, bo
 // Brick load vector f_a = s integral N_a = (s / 8) sum_q |det(2 J_q)| N_a(q): the
 // determinants contracted with the single hats on every axis.
 template <typename T>
-__device__ __forceinline__ void brick_load_from_dets(const T (&det)[8], T s, T (&f)[8]) {
-    T D[2][2][2];
+__device__ __forceinline__ void brick_load_from_dets(const Pair<T> (&det)[2][2], T s, T (&f)[8]) {
+    Pair<T> W[2][2];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) D[q >> 2][(q >> 1) & 1][q & 1] = det[q] < T(0) ? -det[q] : det[q];
-    T V[3][3][3];
-    contract_cross<T, 0, 0, 0>(D, V);
+    for (int q2 = 0; q2 < 2; ++q2) hat_pair(pair_abs(det[q2][0]), pair_abs(det[q2][1]), W[q2][0], W[q2][1]);
 #pragma unroll
-    for (int a = 0; a < 8; ++a) f[a] = s * T(0.125) * V[hb1(a)][hb2(a)][hb3(a)];
+    for (int z = 0; z < 2; ++z) {
+        Pair<T> y[2];
+        hat_pair(W[0][z], W[1][z], y[0], y[1]);
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {
+            const Pair<T> v = hat_in_pair(y[b]);
+            f[hnode(0, b, z)] = s * T(0.125) * pair_lo(v);
+            f[hnode(1, b, z)] = s * T(0.125) * pair_hi(v);
+        }
+    }
 }
 
-// Mixed precision: FP32, except that an element whose max_q det J / min_q det J
-// exceeds `thr` (or with a det J <= 0) takes its determinants from FP64.
+// Mixed precision: FP32, except for the FP64 determinants of a distorted element.
 template <typename S>
 __device__ __forceinline__ bool brick_me_mixed(const S (*xc)[3], float c, float thr, float (&m)[36]) {
-    Vec3<float> e[3][2][2];
-    brick_edges<float, S>(xc, e);
-    Vec3<float> row[3][2][2];
-    brick_jrows(e, row);
-    float det[8];
-    brick_dets(row, det);
-    float dmin = det[0], dmax = det[0];
-#pragma unroll
-    for (int q = 1; q < 8; ++q) {
-        dmin = fminf(dmin, det[q]);
-        dmax = fmaxf(dmax, det[q]);
-    }
-    const bool flagged = !(dmin > 0.f) || dmax > thr * dmin;
-    if (flagged) {
-        Vec3<double> ed[3][2][2];
-        brick_edges<double, S>(xc, ed);
-        Vec3<double> rowd[3][2][2];
-        brick_jrows(ed, rowd);
-        double detd[8];
-        brick_dets(rowd, detd);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) det[q] = (float)detd[q];
-    }
+    Pair<float> det[2][2];
+    const bool flagged = brick_gauss_dets<float, S>(xc, thr, true, det);
     brick_mass_from_dets(det, c, m);
     return flagged;
+}
+template <typename S>
+__device__ __forceinline__ bool brick_me_fp32(const S (*xc)[3], float c, float thr, float (&m)[36]) {
+    BrickRows<float> row;
+    brick_rows<float, S>(xc, row);
+    Pair<float> det[2][2];
+    brick_dets(row, det);
+    brick_mass_from_dets(det, c, m);
+    return brick_distorted(det, thr);
+}
+
+// The final matrix (mass or stiffness) of a distorted element, by eight consecutive
+// lanes of a full warp; all of them get it.
+template <typename S>
+__device__ __forceinline__ void brick_distorted_shared(const S (*xc)[3], float c, bool mass, float (&k)[36]) {
+    float P[8][7];
+    brick_points_shared<S>(xc, c, P);
+    if (mass) {
+        Pair<float> det[2][2];
+        pairs_of_dets(P, det);
+        brick_mass_from_dets(det, c, k);
+    } else {
+        Pair<float> M[2][2][6];
+        pairs_of_points(P, M);
+        brick_contract(M, k);
+    }
 }
 
 // ---------------------------------------------------------------- tetrahedron

@@ -222,7 +222,7 @@ static fem_status closure_range(fem_mesh m, int64_t p0, int64_t p1, cudaStream_t
                                 const std::function<fem_status(const Closure &)> &fn, int *groups,
                                 std::vector<HostClosure> *rec = nullptr, bool *rec_ok = nullptr) {
     Closure cl;
-    fem_status st = build_closure(m, p0, p1, cl, s, m->want_pos || rec != nullptr);
+    fem_status st = build_closure(m, p0, p1, cl, s, m->want_pos || rec != nullptr, false);
     if (st == FEM_ERR_BUDGET && p1 - p0 > 1) {
         cl.reset();
         cudaGetLastError();

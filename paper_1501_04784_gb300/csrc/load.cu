@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(256) k_load(PlanView pv, const S *__restrict__
                     xc[a][2] = xs[ln[a]][2];
                 }
                 if constexpr (NPE == 8) {
-                    T det[8];
+                    Pair<T> det[2][2];
                     brick_gauss_dets<T, S>(xc, thr, MIXED, det);
                     brick_load_from_dets(det, s, fe);
                 } else {

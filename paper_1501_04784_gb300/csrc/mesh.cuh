@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "gather.cuh"
 #include "tile.cuh"
 
 namespace fem {
@@ -29,7 +30,9 @@ struct PlanView {
     const int32_t *own_acc;          // [n_nodes] offset of the owned row in its patch's entries
     const int64_t *own_rowptr;       // [n_nodes] rowptr of the owned row
     const uint8_t *own_hv;           // [n_nodes] 1 if the row's diagonal is summed in FP64 (mixed)
-    const int32_t *cnode_gid;        // [total cnodes] global node id, ascending within a patch
+    const int32_t *cnode_gid;        // [total cnodes] global node id, ascending within a patch (by rank
+                                     // in the locality order where the builds run on gather lists)
+    const int32_t *cnode_rank;       // that rank (gather lists only)
     const int32_t *cnode_own;        // [total cnodes] owned-row index within the patch, or -1
     const int32_t *celem_id;         // [total celems] element id, sorted by (colour, id) in a patch
     const uint8_t *celem_color;      // [total celems]
@@ -49,6 +52,9 @@ struct PlanView {
     int64_t val_off;                 // subtracted from own_rowptr: vals holds the values from
                                      // this CSR position on (a row range of the host pipeline)
     int64_t n_nodes, n_elems, nnz;   // sizes of X, c and vals (bounds checks of the debug build)
+    const GatherPatch *gpatch;       // [n_patches] gather lists (gather.cuh), null without them
+    const uint32_t *gwords;
+    int32_t gzero;
 };
 
 // Marker bit of celem_aidx's FP64-accurate diagonals; scratch accumulators per block.
@@ -63,18 +69,22 @@ struct Closure {
     int n_colors = 0;
     DevBuf<int64_t> patch_elem_ptr, patch_cnode_ptr;
     DevBuf<int32_t> cnode_gid, cnode_own, celem_id;
+    DevBuf<int32_t> cnode_rank;   // with lists: the closure nodes' ranks in the locality order, ascending
     DevBuf<uint8_t> celem_color, celem_pos;
     DevBuf<uint16_t> celem_lnode;
-    DevBuf<uint32_t> celem_aidx;
+    DevBuf<uint32_t> celem_aidx;  // empty when the builds run on the lists
+    GatherLists lists;
     void reset() {
+        lists.free();
         patch_elem_ptr.free(); patch_cnode_ptr.free(); cnode_gid.free(); cnode_own.free(); celem_id.free();
-        celem_color.free(); celem_pos.free(); celem_lnode.free(); celem_aidx.free();
+        celem_color.free(); celem_pos.free(); celem_lnode.free(); celem_aidx.free(); cnode_rank.free();
         p0 = p1 = total_cnodes = total_celems = max_cnodes = max_celems = 0;
         n_colors = 0;
     }
     size_t bytes() const {
         return patch_elem_ptr.bytes() + patch_cnode_ptr.bytes() + cnode_gid.bytes() + cnode_own.bytes() +
-               celem_id.bytes() + celem_color.bytes() + celem_pos.bytes() + celem_lnode.bytes() + celem_aidx.bytes();
+               celem_id.bytes() + celem_color.bytes() + celem_pos.bytes() + celem_lnode.bytes() + celem_aidx.bytes() +
+               lists.bytes() + cnode_rank.bytes();
     }
 };
 
@@ -110,6 +120,7 @@ struct Plan {
         v.own_rowptr = own_rowptr.ptr;
         v.own_hv = own_hv.ptr;
         v.cnode_gid = cl.cnode_gid.ptr;
+        v.cnode_rank = cl.cnode_rank.ptr;
         v.cnode_own = cl.cnode_own.ptr;
         v.celem_id = cl.celem_id.ptr;
         v.celem_color = cl.celem_color.ptr;
@@ -123,6 +134,9 @@ struct Plan {
         v.n_nodes = n_nodes;
         v.n_elems = n_elems;
         v.nnz = nnz;
+        v.gpatch = cl.lists.ready ? cl.lists.patch.ptr : nullptr;
+        v.gwords = cl.lists.words.ptr;
+        v.gzero = cl.lists.zero;
         return v;
     }
     PlanView view() const { return view(full); }
@@ -216,6 +230,7 @@ struct fem_mesh_s {
     fem::DevBuf<int32_t> inc_elem;
     fem::Plan plan;
     bool plan_built = false;  // the patch plan exists (it is built on first use when tiles serve the builds)
+    bool no_lists = false;    // the builds run on the colour-ordered scatter, not on gather lists
     bool want_pos = false;    // closures carry the in-row positions (set by the first backward pass)
     fem::TilePlan tiles;      // element tiles of the scalar operators (tile.cuh)
     // device status word: set by a bounded device-side wait that gave up
@@ -246,6 +261,7 @@ struct fem_mesh_s {
     // pipe is the bound there, so integrating each element once beats recomputing
     // it in every closure that contains it)
     fem::DevBuf<double> ke64;
+    fem::DevBuf<float> xrank;  // [n_nodes][4] FP32 coordinates in locality order (gather builds)
     // host pipeline over row ranges: two device value slots used in turn, the
     // stream their copies to the host run on, chunk_built[j] recorded after the
     // build of the range in slot j, slot_free[j] after its copy out
@@ -269,9 +285,17 @@ fem_status build_plan(fem_mesh m, cudaStream_t s);
 // Frees the host copies of the patch groups and their device slots (the plan changed).
 void drop_group_cache(fem_mesh m);
 // with_pos: the closure carries the in-row positions (the backward pass, the host copies)
-fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaStream_t s, bool with_pos);
+// with_lists: gather lists instead of accumulator targets, where they fit (the full closure)
+fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaStream_t s, bool with_pos,
+                         bool with_lists);
 // From now on the closures carry the in-row positions the backward pass reads.
 fem_status ensure_positions(fem_mesh m, cudaStream_t s);
+// Gather lists of a closure (gather_plan.cu), and whether mesh m's builds may run on them.
+fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s);
+bool wants_lists(fem_mesh m);
+// The full closure's accumulator targets (the colour-ordered scatter): plans mesh m
+// again without gather lists when the builds ran on those.
+fem_status ensure_targets(fem_mesh m, cudaStream_t s);
 // Runs fn over the closure of every patch group (one group covering all patches
 // unless the plan is chunked under the memory budget).
 fem_status for_each_group(fem_mesh m, cudaStream_t s, const std::function<fem_status(const Closure &)> &fn);

@@ -761,6 +761,7 @@ int patch_blocks_per_sm(int npe, int threads) {
 }
 
 fem_status launch_patch(const PatchArgs &a, cudaStream_t s) {
+    if ((a.closure ? *a.closure : a.plan->full).lists.ready) return launch_gather(a, s);
 #define FEM_P(NPE, ACC, S, CT, FU, MX) return launch_patch_t<NPE, ACC, S, CT, FU, MX>(a, s)
     if (!a.mixed) {
         if (a.fused) {
@@ -826,6 +827,7 @@ fem_status batched_config(int npe, bool mixed, const PlanMax &pm, int threads, i
 
 fem_status launch_batched_kernel(const BatchLaunch &bl, cudaStream_t s) {
     if (bl.elastic) return launch_elastic_batched_kernel(bl, s);
+    if (bl.gather) return launch_gather_batched_kernel(bl, s);
     if (bl.tiles) return launch_tile_batched_kernel(bl, s);
 #define FEM_B(NPE, T, MX)                                                                                   \
     k_patch_batched<NPE, T, T, T, MX><<<bl.grid, bl.threads, bl.L.total, s>>>(bl.items, bl.prefix, bl.n, bl.L, \

@@ -79,6 +79,8 @@ struct PatchArgs {
     fem_dtype xd, cd;
     const void *X, *c, *ke;
     void *vals;
+    float *xrank;      // buffer for FP32 coordinates in locality order (gather builds), or null
+    bool x_ordered;    // it holds this call's X already
     float thr;
     int64_t p0, p1;    // patches to run (absolute numbers; those the closure holds)
     int64_t val_off;   // vals holds the CSR values from this position on (scalar operators)
@@ -99,6 +101,27 @@ struct PlanMax {
         max_cnodes = std::max(max_cnodes, P.max_cnodes);
     }
 };
+
+// Gather assembly (gather.cu): shared memory of a block and the largest patch sizes
+// over the plans a launch covers.
+struct GatherSmem {
+    size_t tab, rowd, bad, ke, xs, cs, gid, eid, total;
+    int n_bad;
+};
+struct GatherMax {
+    int64_t max_acc = 0, max_own = 0, max_cnodes = 0, max_celems = 0;
+    void add(const Plan &P) {
+        max_acc = std::max(max_acc, P.max_acc);
+        max_own = std::max(max_own, P.max_own);
+        max_cnodes = std::max(max_cnodes, P.max_cnodes);
+        max_celems = std::max(max_celems, P.max_celems);
+    }
+};
+GatherSmem gather_smem_layout(const GatherMax &g, int npe, bool fused, size_t accsize, size_t xsize, size_t csize);
+fem_status launch_gather(const PatchArgs &a, cudaStream_t s);
+int gather_blocks_per_sm(int npe, int threads);
+// The plan's nodes' FP32 coordinates in locality order, 16 bytes each.
+fem_status launch_order_x(const Plan &P, const float *X, float *xrank, cudaStream_t s);
 
 // One mesh of a batched build.
 struct BatchItem {
@@ -152,6 +175,10 @@ struct BatchLaunch {
     WaitCtl wait{nullptr, WAIT_SPINS_DEFAULT, 0};
     bool elastic = false;  // the elasticity operator's kernel (elastic.cu)
     bool win = false;      // its row-window variant (the FP64 blocks outgrow shared memory)
+    bool gather = false;   // the gather kernel (gather.cu) over gpatch
+    const GatherPatch *gpatch = nullptr;  // every patch of the batch, its mesh's index in `pad`
+    int64_t n_work = 0;
+    GatherSmem gl{};
     bool tiles = false;    // the element-tile kernel (tile.cu) over titems
     const TileBatchItem *titems = nullptr;
     const int64_t *bprefix = nullptr;  // tiles: prefix sums of the meshes' border rows (the combine's work)
@@ -163,6 +190,12 @@ struct BatchLaunch {
 // and at most `blocks_per_sm` blocks per SM (0 = as many as fit).
 fem_status batched_config(int npe, bool mixed, const PlanMax &pm, int threads, int blocks_per_sm, BatchLaunch *out);
 fem_status launch_batched_kernel(const BatchLaunch &bl, cudaStream_t s);
+
+fem_status gather_batched_config(int npe, bool mixed, const GatherMax &gm, int threads, int blocks_per_sm,
+                                 BatchLaunch *out);
+fem_status launch_gather_batched_kernel(const BatchLaunch &bl, cudaStream_t s);
+// The batch's patches in one table: out[w] = src[w], its mesh's index in `pad`.
+fem_status launch_gather_table(const GatherPatch *src, int64_t n, int mesh, GatherPatch *out, cudaStream_t s);
 
 fem_status launch_integrate(const IntegrateArgs &a, cudaStream_t s);
 

@@ -32,22 +32,20 @@ __device__ __forceinline__ Pair<float> operator+(Pair<float> a, Pair<float> b) {
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
-__device__ __forceinline__ Pair<float> operator*(Pair<float> a, Pair<float> b) {
-    Pair<float> r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
 __device__ __forceinline__ Pair<float> pfma(Pair<float> a, Pair<float> b, Pair<float> c) {
     Pair<float> r;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
     return r;
 }
+// a b + 0: a plain mul.rn.f32x2 followed by an addition was fused by the assembler in
+// one kernel and not in another, and builds have to agree bit for bit.
+__device__ __forceinline__ Pair<float> operator*(Pair<float> a, Pair<float> b) { return pfma(a, b, Pair<float>{0ull}); }
 __device__ __forceinline__ Pair<float> operator-(Pair<float> a, Pair<float> b) {
     Pair<float> r;
     asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
-__device__ __forceinline__ Pair<float> operator-(Pair<float> a) { return a * pair(-1.f, -1.f); }
+__device__ __forceinline__ Pair<float> operator-(Pair<float> a) { return Pair<float>{0ull} - a; }
 
 __device__ __forceinline__ Pair<double> pair(double lo, double hi) { return {lo, hi}; }
 __device__ __forceinline__ double pair_lo(Pair<double> p) { return p.x; }

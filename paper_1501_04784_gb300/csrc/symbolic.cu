@@ -675,14 +675,21 @@ __global__ void k_cnode_pairs(const uint64_t *ckeys, int64_t nce, int npe, const
 }
 
 __global__ void k_cnode_own(const uint64_t *cn_keys, int64_t ncn, int64_t p0, const int32_t *node_patch,
-                            const int32_t *own_idx, int32_t *gid, int32_t *own) {
+                            const int32_t *own_idx, const int32_t *by_rank, int32_t *gid, int32_t *own, int32_t *rank) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < ncn; j += (int64_t)gridDim.x * blockDim.x) {
         const uint64_t k = cn_keys[j];
-        const int32_t g = (int32_t)(k & 0xffffffffull);
+        const int32_t key = (int32_t)(k & 0xffffffffull), g = by_rank ? by_rank[key] : key;
         const int32_t p = (int32_t)(p0 + (int64_t)(k >> 32));
         gid[j] = g;
         own[j] = node_patch[g] == p ? own_idx[g] : -1;
+        if (rank) rank[j] = key;
     }
+}
+
+// rank[order[k]] = k.
+__global__ void k_invert(const int32_t *order, int64_t n, int32_t *rank) {
+    for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x)
+        rank[order[k]] = (int32_t)k;
 }
 
 // Per closure element: id, colour, closure-local node indices (binary search in
@@ -719,14 +726,16 @@ __device__ __forceinline__ int pair_position(const int32_t (&g)[NPE], const int6
 }
 
 template <int NPE>
-// One block per patch: the patch's closure-node ids (ascending) are staged in
-// shared memory, so that the closure-local index of each element node is a
+// One block per patch: the patch's closure-node ids (ascending; with `rank`, the
+// nodes' ranks in the locality order) are staged in shared memory, so that the closure-local index of each element node is a
 // binary search there rather than a chain of dependent global loads.  The in-row
-// positions (pos) are written only when the closures carry them (pos non-null).
+// positions (pos) and the targets (aidx) are written only when the closures carry
+// them (non-null).
 __global__ void __launch_bounds__(256, 3) k_celem_fill(const uint64_t *ckeys, int64_t np_, const int32_t *__restrict__ E,
                              const uint64_t *cn_keys, const int64_t *pc_ptr, const int64_t *__restrict__ rowptr,
                              const int32_t *__restrict__ col, int pos_stride, OwnTables ot, int32_t *celem_id,
-                             uint8_t *celem_color, uint16_t *lnode, uint8_t *pos, uint16_t *aidx) {
+                             uint8_t *celem_color, uint16_t *lnode, uint8_t *pos, uint16_t *aidx,
+                             const int32_t *__restrict__ rank) {
     extern __shared__ int32_t cn_gid[];
     const int64_t nce = ot.pe_ptr[np_];
   for (int64_t pb = blockIdx.x; pb < np_; pb += gridDim.x) {
@@ -745,15 +754,17 @@ __global__ void __launch_bounds__(256, 3) k_celem_fill(const uint64_t *ckeys, in
 #pragma unroll
         for (int a = 0; a < NPE; ++a) {
             g[a] = E[e * NPE + a];
+            const int32_t key = rank ? rank[g[a]] : g[a];
             int lo = 0, hi = ncn;
             while (lo < hi) {
                 const int mid = (lo + hi) >> 1;
-                if (cn_gid[mid] < g[a]) lo = mid + 1; else hi = mid;
+                if (cn_gid[mid] < key) lo = mid + 1; else hi = mid;
             }
             if (a & 1) lw[a >> 1] |= (uint32_t)lo << 16; else lw[a >> 1] = (uint32_t)lo;
         }
         if constexpr (NPE == 8) reinterpret_cast<uint4 *>(lnode)[i] = make_uint4(lw[0], lw[1], lw[2], lw[3]);
         else reinterpret_cast<uint2 *>(lnode)[i] = make_uint2(lw[0], lw[1]);
+        if (!pos && !aidx) continue;  // the builds run on gather lists
         const int64_t gp = ot.p0 + (int64_t)p;
         const int64_t nb = ot.patch_node_ptr[gp];
         // Each element node x as a row: its start and length, and the row's
@@ -803,6 +814,7 @@ __global__ void __launch_bounds__(256, 3) k_celem_fill(const uint64_t *ckeys, in
                     else t = (uint32_t)((ra ? base[a] : base[b]) + ps);
                 }
                 // word q/2 of element i, low half for even q
+                if (!aidx) continue;
                 if (q & 1) aidx32[(int64_t)(q >> 1) * nce + i] = alo | ((t & 0xffffu) << 16);
                 else alo = t & 0xffffu;
             }
@@ -1108,13 +1120,13 @@ __global__ void __launch_bounds__(256) k_patch_celems(const int64_t *pn_ptr, int
 }
 
 // Closure nodes of each patch (one block per patch): the nodes of the patch's
-// closure elements, made unique in a shared-memory hash set and sorted
-// ascending, written to tmp from the patch's offset (npe slots per closure
+// closure elements (with `rank`, their ranks in the locality order), made unique in
+// a shared-memory hash set and sorted ascending, written to tmp from the patch's offset (npe slots per closure
 // element) with their number in cnt.
 template <int NPE>
 __global__ void __launch_bounds__(256) k_patch_cnodes(const uint64_t *ckeys, const int64_t *pe_ptr, int64_t np_,
-                                                      const int32_t *__restrict__ E, int hsize, uint32_t *tmp,
-                                                      int64_t *cnt, int *overflow) {
+                                                      const int32_t *__restrict__ E, const int32_t *__restrict__ rank,
+                                                      int hsize, uint32_t *tmp, int64_t *cnt, int *overflow) {
     extern __shared__ __align__(16) unsigned char cn_smem[];
     uint32_t *table = reinterpret_cast<uint32_t *>(cn_smem);  // [hsize], then the sort keys
     uint32_t *list = reinterpret_cast<uint32_t *>(cn_smem + (size_t)hsize * sizeof(uint32_t));  // [hsize]
@@ -1125,9 +1137,10 @@ __global__ void __launch_bounds__(256) k_patch_cnodes(const uint64_t *ckeys, con
         __syncthreads();
         const int64_t b = pe_ptr[p];
         const int n = (int)(pe_ptr[p + 1] - b) * NPE;
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            set_insert(table, hsize, (uint32_t)E[(int64_t)(uint32_t)ckeys[b + i / NPE] * NPE + i % NPE], list, &n_set,
-                       &s_full);
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const int32_t g = E[(int64_t)(uint32_t)ckeys[b + i / NPE] * NPE + i % NPE];
+            set_insert(table, hsize, (uint32_t)(rank ? rank[g] : g), list, &n_set, &s_full);
+        }
         __syncthreads();
         if (s_full) {
             if (threadIdx.x == 0) {
@@ -1180,7 +1193,8 @@ __global__ void __launch_bounds__(512) k_patch_color_order(const uint64_t *ckeys
     }
 }
 
-fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaStream_t s, bool with_pos) {
+fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaStream_t s, bool with_pos,
+                         bool with_lists) {
     Arena &ar = m->arena;
     Plan &P = m->plan;
     const int64_t npe = m->npe;
@@ -1363,7 +1377,15 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         std::swap(ckeys.arena, ck2.arena);
     }
 
-    // ---- closure nodes of each patch
+    // ---- closure nodes of each patch: ascending ids, or for the gather kernels
+    // ascending ranks in the locality order, so that a patch's own nodes are one run
+    // and its neighbours' a few
+    DevBuf<int32_t> rank;
+    if (with_lists) {
+        FEM_TRY(rank.alloc(ar, m->n_nodes, "node ranks"));
+        k_invert<<<grid_for(m->n_nodes), TPB, 0, s>>>(P.own_row.ptr, m->n_nodes, rank.ptr);
+        FEM_LAUNCHED("k_invert");
+    }
     DevBuf<uint64_t> cnkeys;
     int64_t ncn = 0;
     bool cn_done = false;
@@ -1384,7 +1406,8 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         int per_sm = 1;
         FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, smem));
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np_, (int64_t)num_sms() * std::max(per_sm, 1)));
-        f<<<grid, 256, smem, s>>>(ckeys.ptr, cl.patch_elem_ptr.ptr, np_, m->E, hsize, ntmp.ptr, cnt.ptr, ovf.ptr);
+        f<<<grid, 256, smem, s>>>(ckeys.ptr, cl.patch_elem_ptr.ptr, np_, m->E, rank.ptr, hsize, ntmp.ptr, cnt.ptr,
+                                  ovf.ptr);
         FEM_LAUNCHED("k_patch_cnodes");
         int h_ovf = 0;
         std::vector<int64_t> h_cnt(np_), h_off(np_ + 1, 0);
@@ -1405,6 +1428,8 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         }
     }
     if (!cn_done) {
+        with_lists = false;  // a closure this large is out of the gather kernels' range
+        rank.free();
         DevBuf<uint64_t> pairs;
         FEM_TRY(pairs.alloc(ar, nce * npe, "closure node pairs"));
         k_cnode_pairs<<<grid_for(nce * npe), TPB, 0, s>>>(ckeys.ptr, nce, (int)npe, m->E, pairs.ptr);
@@ -1417,8 +1442,10 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
     FEM_LAUNCHED("k_segment_ptr(cnodes)");
     FEM_TRY(cl.cnode_gid.alloc(ar, ncn, "cnode gid"));
     FEM_TRY(cl.cnode_own.alloc(ar, ncn, "cnode own"));
-    k_cnode_own<<<grid_for(ncn), TPB, 0, s>>>(cnkeys.ptr, ncn, p0, P.node_patch.ptr, P.own_idx.ptr, cl.cnode_gid.ptr,
-                                              cl.cnode_own.ptr);
+    if (with_lists) FEM_TRY(cl.cnode_rank.alloc(ar, ncn, "cnode ranks"));
+    k_cnode_own<<<grid_for(ncn), TPB, 0, s>>>(cnkeys.ptr, ncn, p0, P.node_patch.ptr, P.own_idx.ptr,
+                                              rank.ptr ? P.own_row.ptr : nullptr, cl.cnode_gid.ptr, cl.cnode_own.ptr,
+                                              cl.cnode_rank.ptr);
     FEM_LAUNCHED("k_cnode_own");
 
     // ---- per closure element data
@@ -1426,10 +1453,8 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
     FEM_TRY(cl.celem_color.alloc(ar, nce, "celem colour"));
     FEM_TRY(cl.celem_lnode.alloc(ar, nce * npe, "celem local nodes"));
     if (with_pos) FEM_TRY(cl.celem_pos.alloc(ar, nce * P.pos_stride, "celem positions"));
-    FEM_TRY(cl.celem_aidx.alloc(ar, nce * (m->np / 2), "celem accumulator targets"));
     const OwnTables ot{P.node_patch.ptr,     P.own_idx.ptr, P.own_acc.ptr,          P.patch_node_ptr.ptr,
                        P.own_hv.ptr,         cl.patch_elem_ptr.ptr, p0, (int32_t)P.max_acc};
-    uint16_t *aidx16 = reinterpret_cast<uint16_t *>(cl.celem_aidx.ptr);
     FEM_CUDA(cudaMemcpyAsync(h_pc.data(), cl.patch_cnode_ptr.ptr, (np_ + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     FEM_CUDA(cudaStreamSynchronize(s));
     for (int64_t p = 0; p < np_; ++p) cl.max_cnodes = std::max(cl.max_cnodes, h_pc[p + 1] - h_pc[p]);
@@ -1437,24 +1462,53 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         set_error("a patch touches %lld nodes; at most 32768 are supported", (long long)cl.max_cnodes);
         return FEM_ERR_UNSUPPORTED;
     }
-    {
+    auto fill = [&]() -> fem_status {
         const size_t smem = (size_t)std::max<int64_t>(cl.max_cnodes, 1) * sizeof(int32_t);
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np_, (int64_t)num_sms() * 8));
-        if (npe == 8) {
-            FEM_CUDA(cudaFuncSetAttribute(k_celem_fill<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            k_celem_fill<8><<<grid, TPB, smem, s>>>(ckeys.ptr, np_, m->E, cnkeys.ptr, cl.patch_cnode_ptr.ptr,
-                                                    m->rowptr.ptr, m->col.ptr, P.pos_stride, ot, cl.celem_id.ptr,
-                                                    cl.celem_color.ptr, cl.celem_lnode.ptr,
-                                                    with_pos ? cl.celem_pos.ptr : nullptr, aidx16);
-        } else {
-            FEM_CUDA(cudaFuncSetAttribute(k_celem_fill<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-            k_celem_fill<4><<<grid, TPB, smem, s>>>(ckeys.ptr, np_, m->E, cnkeys.ptr, cl.patch_cnode_ptr.ptr,
-                                                    m->rowptr.ptr, m->col.ptr, P.pos_stride, ot, cl.celem_id.ptr,
-                                                    cl.celem_color.ptr, cl.celem_lnode.ptr,
-                                                    with_pos ? cl.celem_pos.ptr : nullptr, aidx16);
-        }
+        auto f = npe == 8 ? k_celem_fill<8> : k_celem_fill<4>;
+        FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        f<<<grid, TPB, smem, s>>>(ckeys.ptr, np_, m->E, cnkeys.ptr, cl.patch_cnode_ptr.ptr, m->rowptr.ptr, m->col.ptr,
+                                  P.pos_stride, ot, cl.celem_id.ptr, cl.celem_color.ptr, cl.celem_lnode.ptr,
+                                  with_pos ? cl.celem_pos.ptr : nullptr,
+                                  reinterpret_cast<uint16_t *>(cl.celem_aidx.ptr), rank.ptr);
         FEM_LAUNCHED("k_celem_fill");
+        return FEM_OK;
+    };
+    if (with_lists) {
+        // gather lists instead of accumulator targets, unless the patches are out of
+        // the gather kernels' range or the budget refuses them
+        FEM_TRY(fill());
+        const fem_status st = build_gather_lists(m, cl, s);
+        if (st != FEM_OK && st != FEM_ERR_BUDGET) return st;
+        if (cl.lists.ready) {
+            // coordinates in locality order, filled by each mixed build (refused by the
+            // budget: the builds gather them from X)
+            if (m->xrank.n < 4 * (size_t)m->n_nodes && m->xrank.alloc(ar, 4 * (size_t)m->n_nodes, "ordered X") != FEM_OK)
+                cudaGetLastError();
+            return FEM_OK;
+        }
+        cl.lists.free();
+        cl.cnode_rank.free();
+        cudaGetLastError();
     }
+    FEM_TRY(cl.celem_aidx.alloc(ar, nce * (m->np / 2), "celem accumulator targets"));
+    return fill();
+}
+
+// Gather lists serve the scalar operators' builds; the fused FP64 form and the
+// kernels' test modes run on the colour-ordered scatter.
+bool wants_lists(fem_mesh m) {
+    return m->opt.operator_kind != 2 && !m->opt.fp64_fused && !m->opt.debug_stall && !m->no_lists;
+}
+
+fem_status ensure_targets(fem_mesh m, cudaStream_t s) {
+    if (!m->plan_built || m->plan.chunked || !m->plan.full.lists.ready) return FEM_OK;
+    m->no_lists = true;
+    batch_forget(m);
+    m->plan_built = false;
+    ArenaKeep keep(m->arena);
+    FEM_TRY(build_plan(m, s));
+    m->plan_built = true;
     return FEM_OK;
 }
 
@@ -1507,7 +1561,7 @@ static fem_status plan_groups(fem_mesh m, cudaStream_t s) {
     for (;;) {
         Closure cl;
         // (with the host copies, the groups are recorded with their in-row positions)
-        fem_status st = build_closure(m, 0, std::min(G, P.n_patches), cl, s, m->want_pos || m->opt.group_cache);
+        fem_status st = build_closure(m, 0, std::min(G, P.n_patches), cl, s, m->want_pos || m->opt.group_cache, false);
         if (st == FEM_OK) break;
         cl.reset();
         cudaGetLastError();
@@ -1543,10 +1597,18 @@ static fem_status build_plan_cap(fem_mesh m, cudaStream_t s, int64_t cap_in) {
     drop_group_cache(m);
     // the elasticity operator holds a 3x3 block per node pair: fewer pairs fit
     const bool elastic = m->opt.operator_kind == 2;
-    // (defaults measured on the 1M-brick and 3.07M-tet workloads)
-    int64_t cap_entries = cap_in > 0 ? cap_in
-                                     : m->opt.patch_entries > 0 ? m->opt.patch_entries
-                                                                : (elastic ? (m->npe == 8 ? 4096 : 1536) : 8192);
+    // Defaults, measured.  Gather lists: two 256-thread blocks of bricks share an SM up
+    // to about 500 closure elements a patch, also two rounds of a block (1M bricks:
+    // 171 us at 3,072 entries, 180 at 2,688, 199 at 4,096 with one block an SM).
+    // Meshes of up to 2^18 nodes take fewer: their odd shapes have larger closures, and
+    // a batch's launch is sized by the largest of all (512 meshes: 2.71 ms at 2,816,
+    // 3.31 at 3,072).  Tetrahedra: 152 us at 1,024, 173 at 1,280 (3.07M).
+    int64_t cap_entries = cap_in > 0 ? cap_in : m->opt.patch_entries;
+    if (cap_entries <= 0) {
+        if (elastic) cap_entries = m->npe == 8 ? 4096 : 1536;
+        else if (!wants_lists(m)) cap_entries = 8192;
+        else cap_entries = m->npe == 4 ? 1024 : N < (1 << 18) ? 2816 : 3072;
+    }
     if (cap_entries < 2 * (int64_t)m->max_row_len) cap_entries = 2 * (int64_t)m->max_row_len;
     P.cap_entries = cap_entries;
     int64_t cap_eff = cap_entries - m->max_row_len;
@@ -1592,7 +1654,7 @@ static fem_status build_plan_cap(fem_mesh m, cudaStream_t s, int64_t cap_in) {
             const int64_t smem = 36 * (cap_entries + 32) + 16384;
             per_sm = (int)std::max<int64_t>(1, std::min<int64_t>(per_sm, (228 * 1024) / (smem + 1024)));
         } else {
-            per_sm = patch_blocks_per_sm(m->npe, threads);
+            per_sm = wants_lists(m) ? gather_blocks_per_sm(m->npe, threads) : patch_blocks_per_sm(m->npe, threads);
         }
         wave = (int64_t)num_sms() * per_sm;
     }
@@ -1665,7 +1727,7 @@ static fem_status build_plan_cap(fem_mesh m, cudaStream_t s, int64_t cap_in) {
     }
 
     // closures of all patches, unless the budget refuses them
-    fem_status st = build_closure(m, 0, npatch, P.full, s, m->want_pos);
+    fem_status st = build_closure(m, 0, npatch, P.full, s, m->want_pos, wants_lists(m));
     if (st == FEM_ERR_BUDGET) {
         P.full.reset();
         cudaGetLastError();
