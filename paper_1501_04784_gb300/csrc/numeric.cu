@@ -55,6 +55,18 @@ __device__ __forceinline__ void load_packed(const T *__restrict__ src, T (&kv)[N
 // in one coalesced stream per block, which measured faster for them.
 static constexpr int INT_THREADS = 128;
 
+// Threads of a block.  FP64: one warp, so that no warp waits for another's stores
+// (1M bricks 1.900 -> 1.886 ms), and few elements spread over the most SMs: the FP64
+// pipe takes a warp instruction every 16 cycles of an SM whatever its lanes do, so the
+// integration of 8,000 bricks takes as long as the SM with the most warps, four in
+// blocks of 128 on 63 SMs but two in 250 blocks of 32 (their FP64 build 51.9 -> 47.4 us).
+// FP32: 128, fewer where that spreads few elements.
+static int integrate_threads(int64_t nel, bool fp64) {
+    int t = fp64 ? 32 : INT_THREADS;
+    while (t > 32 && cdiv(nel, t) < 4 * (int64_t)num_sms()) t /= 2;
+    return t;
+}
+
 template <int NPE, typename T>
 __host__ __device__ constexpr bool int_direct() { return NPE == 8 && sizeof(T) == 4; }
 template <int NPE, typename T>
@@ -76,8 +88,10 @@ __global__ void __launch_bounds__(INT_THREADS, (int_min_blocks<NPE, T>())) k_int
     extern __shared__ __align__(16) unsigned char int_smem[];
     T *st = reinterpret_cast<T *>(int_smem);
     unsigned flagged = 0;
-    for (int64_t e0 = (int64_t)blockIdx.x * INT_THREADS; e0 < nel; e0 += (int64_t)gridDim.x * INT_THREADS) {
+    const int nthr = blockDim.x;
+    for (int64_t e0 = (int64_t)blockIdx.x * nthr; e0 < nel; e0 += (int64_t)gridDim.x * nthr) {
         const int64_t e = e0 + threadIdx.x;
+        bool distorted = false;  // a brick whose FP32 matrix is replaced below
         if (e < nel) {
             int32_t g[NPE];
             load_ids<NPE>(E, e, g);
@@ -89,8 +103,13 @@ __global__ void __launch_bounds__(INT_THREADS, (int_min_blocks<NPE, T>())) k_int
                 xc[a][2] = __ldg(X + 3 * (int64_t)g[a] + 2);
             }
             T k[NP];
-            flagged += element_matrix<NPE, T, S, MIXED>(xc, __ldg(c + e), thr, mode, k) ? 1u : 0u;
-            if (status && !isfinite(k[0])) atomicOr(status, STATUS_NONFINITE);
+            if constexpr (int_direct<NPE, T>()) {
+                distorted = element_matrix_fast<NPE, T, S, MIXED>(xc, __ldg(c + e), thr, mode, k);
+                flagged += distorted;
+            } else {
+                flagged += element_matrix<NPE, T, S, MIXED>(xc, __ldg(c + e), thr, mode, k) ? 1u : 0u;
+            }
+            if (status && !distorted && !isfinite(k[0])) atomicOr(status, STATUS_NONFINITE);
             if constexpr (int_direct<NPE, T>()) {
                 store_row16<NP>(reinterpret_cast<float *>(ke_out + e * NP), k);
             } else {
@@ -98,11 +117,33 @@ __global__ void __launch_bounds__(INT_THREADS, (int_min_blocks<NPE, T>())) k_int
                 for (int p = 0; p < NP; ++p) st[threadIdx.x * LD + p] = k[p];
             }
         }
+        if constexpr (int_direct<NPE, T>()) {
+            // distorted elements of the warp: four at a time, eight lanes each (the last
+            // again where there are fewer)
+            for (unsigned fm = __ballot_sync(0xffffffffu, distorted); fm;) {
+                int src = __ffs(fm) - 1;
+                for (int k = 0; k < 4 && fm; ++k, fm &= fm - 1)
+                    if (k <= (int)(threadIdx.x & 31) >> 3) src = __ffs(fm) - 1;
+                const int64_t f = e - (threadIdx.x & 31) + src;
+                int32_t g[NPE];
+                load_ids<NPE>(E, f, g);
+                S xc[NPE][3];
+#pragma unroll
+                for (int a = 0; a < NPE; ++a)
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) xc[a][d] = __ldg(X + 3 * (int64_t)g[a] + d);
+                T k[NP];
+                brick_distorted_shared<S>(xc, (float)__ldg(c + f), (mode & OP_MASS) != 0, k);
+                if (status && !isfinite(k[0])) atomicOr(status, STATUS_NONFINITE);
+                __syncwarp();  // the FP32 row was stored by another lane
+                if ((threadIdx.x & 7) == 0) store_row16<NP>(reinterpret_cast<float *>(ke_out + f * NP), k);
+            }
+        }
         if constexpr (!int_direct<NPE, T>()) {
             __syncthreads();
-            const int nb = (int)min((int64_t)INT_THREADS, nel - e0);
+            const int nb = (int)min((int64_t)nthr, nel - e0);
             T *out = ke_out + e0 * NP;
-            for (int idx = threadIdx.x; idx < nb * NP; idx += INT_THREADS) out[idx] = st[(idx / NP) * LD + idx % NP];
+            for (int idx = threadIdx.x; idx < nb * NP; idx += nthr) out[idx] = st[(idx / NP) * LD + idx % NP];
             __syncthreads();
         }
     }
@@ -608,15 +649,16 @@ template <int NPE, typename T, typename S, typename CT, bool MIXED>
 static fem_status launch_integrate_t(const int32_t *E, int64_t nel, const void *X, const void *c, void *ke, float thr,
                                      unsigned mode, unsigned long long *nflag, int *status, cudaStream_t s) {
     constexpr int NP = ElemTraits<NPE>::NP;
-    const size_t smem = int_direct<NPE, T>() ? 0 : (size_t)INT_THREADS * (NP + 1) * sizeof(T);
+    const int threads = integrate_threads(nel, sizeof(T) == 8);
+    const size_t smem = int_direct<NPE, T>() ? 0 : (size_t)threads * (NP + 1) * sizeof(T);
     auto f = k_integrate<NPE, T, S, CT, MIXED>;
     if (smem) FEM_TRY(set_smem(f, smem));
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, INT_THREADS, smem));
+    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem));
     if (per_sm < 1) per_sm = 1;
-    const int64_t tiles = cdiv(nel, INT_THREADS);
+    const int64_t tiles = cdiv(nel, threads);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)num_sms() * per_sm));
-    f<<<grid, INT_THREADS, smem, s>>>(E, nel, (const S *)X, (const CT *)c, (T *)ke, thr, mode, nflag, status);
+    f<<<grid, threads, smem, s>>>(E, nel, (const S *)X, (const CT *)c, (T *)ke, thr, mode, nflag, status);
     FEM_LAUNCHED("k_integrate");
     return FEM_OK;
 }
