@@ -150,4 +150,13 @@ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 int num_sms();
 
+// cudaOccupancyMaxActiveBlocksPerMultiprocessor with its answers remembered: they depend
+// on the kernel, the device and the launch shape alone, and the query costs some 4 us
+// of every launch.  At most a few hundred shapes are kept.
+cudaError_t resident_blocks_of(int *n, const void *kernel, int threads, size_t smem);
+template <typename F>
+cudaError_t resident_blocks(int *n, F kernel, int threads, size_t smem) {
+    return resident_blocks_of(n, reinterpret_cast<const void *>(kernel), threads, smem);
+}
+
 }  // namespace fem

@@ -417,7 +417,7 @@ static fem_status launch_elastic_patch_t(const PatchArgs &a, cudaStream_t s) {
     FEM_TRY(el_set_smem(f, L.total));
     const int threads = std::min(elastic_threads(NPE, a.threads), elastic_max_threads<NPE, AccT>());
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, L.total));
+    FEM_CUDA(resident_blocks(&per_sm, f, threads, L.total));
     if (per_sm < 1) {
         set_error("elastic patch kernel cannot be resident with %d threads and %zu bytes of shared memory", threads,
                   L.total);
@@ -530,7 +530,7 @@ template <int NPE, typename T, typename S, typename CT, bool MIXED>
 static fem_status launch_elastic_integrate_t(const IntegrateArgs &a, cudaStream_t s) {
     auto f = k_elastic_integrate<NPE, T, S, CT, MIXED>;
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, EL_INT_THREADS, 0));
+    FEM_CUDA(resident_blocks(&per_sm, f, EL_INT_THREADS, 0));
     if (per_sm < 1) per_sm = 1;
     const int64_t tiles = cdiv(a.nel, EL_INT_THREADS / NPE);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)num_sms() * per_sm * 4));

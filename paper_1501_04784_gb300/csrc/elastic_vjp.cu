@@ -528,7 +528,7 @@ static fem_status launch_elastic_vjp_t(fem_mesh m, const Closure &cl, const void
     auto f = staged ? k_elastic_vjp_elem<NPE, T, S, CT> : k_elastic_vjp<NPE, T, S, CT>;
     FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, L.total));
+    FEM_CUDA(resident_blocks(&per_sm, f, 256, L.total));
     if (per_sm < 1) {
         set_error("elasticity backward kernel cannot be resident with %zu bytes of shared memory", L.total);
         return FEM_ERR_UNSUPPORTED;

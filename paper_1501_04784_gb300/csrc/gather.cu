@@ -482,8 +482,10 @@ fem_status launch_order_x(const Plan &P, const float *X, float *xrank, cudaStrea
 // order first, so that the patches copy them in runs of 16-byte rows instead of three
 // 4-byte words a node at its id: 1M permuted bricks 175.7 -> 171.3 us with the extra
 // launch, 27M in natural numbering (whose ids come in runs by themselves) 3.84 -> 3.89
-// ms.  Batches, mostly of smaller meshes, copy by id (512 meshes: the extra pass 0.13 ms).
-static constexpr int64_t XRANK_MIN = 16384;
+// ms.  Below, the launch costs more than it saves (80,000 bricks' mass matrix and load
+// vector 43 us with it, 37 without).  Batches copy by id too (512 meshes: the extra
+// pass 0.13 ms).
+static constexpr int64_t XRANK_MIN = 1 << 18;
 
 GatherSmem gather_smem_layout(const GatherMax &g, int npe, bool fused, size_t accsize, size_t xsize, size_t csize) {
     GatherSmem L{};
@@ -514,7 +516,7 @@ GatherSmem gather_smem_layout(const GatherMax &g, int npe, bool fused, size_t ac
 template <typename F>
 static fem_status resident(F *f, int threads, size_t bytes, int *per_sm) {
     FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, f, threads, bytes));
+    FEM_CUDA(resident_blocks(per_sm, f, threads, bytes));
     if (*per_sm < 1) {
         set_error("the gather kernel cannot be resident with %d threads and %zu bytes of shared memory", threads, bytes);
         return FEM_ERR_UNSUPPORTED;

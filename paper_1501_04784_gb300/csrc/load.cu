@@ -136,7 +136,7 @@ static fem_status launch_load_t(fem_mesh m, const Closure &cl, const void *X, co
     auto f = k_load<NPE, T, S, CT, MIXED, NC>;
     FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, L.total));
+    FEM_CUDA(resident_blocks(&per_sm, f, 256, L.total));
     if (per_sm < 1) {
         set_error("load-vector kernel cannot be resident with %zu bytes of shared memory", L.total);
         return FEM_ERR_UNSUPPORTED;

@@ -654,7 +654,7 @@ static fem_status launch_integrate_t(const int32_t *E, int64_t nel, const void *
     auto f = k_integrate<NPE, T, S, CT, MIXED>;
     if (smem) FEM_TRY(set_smem(f, smem));
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem));
+    FEM_CUDA(resident_blocks(&per_sm, f, threads, smem));
     if (per_sm < 1) per_sm = 1;
     const int64_t tiles = cdiv(nel, threads);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)num_sms() * per_sm));
@@ -751,7 +751,7 @@ static fem_status launch_patch_t(const PatchArgs &a, cudaStream_t s) {
     FEM_TRY(set_smem(f, L.total));
     const int threads = a.threads;
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, L.total));
+    FEM_CUDA(resident_blocks(&per_sm, f, threads, L.total));
     if (per_sm < 1) {
         set_error("patch kernel cannot be resident with %d threads and %zu bytes of shared memory", threads, L.total);
         return FEM_ERR_UNSUPPORTED;
@@ -774,7 +774,7 @@ static fem_status launch_patch_t(const PatchArgs &a, cudaStream_t s) {
         if (Lp.total + fpa.sharedSizeBytes <= (size_t)max_optin) {
             FEM_TRY(set_smem(fp, Lp.total));
             int per_pf = 0;
-            FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_pf, fp, threads, Lp.total));
+            FEM_CUDA(resident_blocks(&per_pf, fp, threads, Lp.total));
             if (a.blocks_per_sm > 0 && a.blocks_per_sm < per_pf) per_pf = a.blocks_per_sm;
             if (per_pf >= per_sm) {
                 fp<<<grid, threads, Lp.total, s>>>(pv, (const S *)a.X, (const CT *)a.c, (AccT *)a.vals, a.thr, q0, q1,

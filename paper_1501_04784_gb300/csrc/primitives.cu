@@ -3,6 +3,8 @@
 #include <cstdarg>
 #include <cstring>
 #include <iterator>
+#include <mutex>
+#include <tuple>
 
 #include "common.cuh"
 
@@ -170,6 +172,27 @@ bool Arena::uncarve(void *p, size_t size) {
         return true;
     }
     return false;
+}
+
+cudaError_t resident_blocks_of(int *n, const void *kernel, int threads, size_t smem) {
+    using Key = std::tuple<const void *, int, int, size_t>;
+    static std::mutex mu;
+    static std::map<Key, int> known;
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const Key key{kernel, dev, threads, smem};
+    std::lock_guard<std::mutex> lock(mu);
+    const auto it = known.find(key);
+    if (it != known.end()) {
+        *n = it->second;
+        return cudaSuccess;
+    }
+    const cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, kernel, threads, smem);
+    if (q != cudaSuccess || *n < 1) return q;  // (asked again next time)
+    if (known.size() >= 512) known.clear();
+    known[key] = *n;
+    return cudaSuccess;
 }
 
 int num_sms() {

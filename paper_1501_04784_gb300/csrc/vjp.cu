@@ -534,7 +534,7 @@ static fem_status launch_vjp_t(fem_mesh m, const Closure &cl, const void *X, con
     auto f = m->opt.operator_kind == 1 ? k_vjp<NPE, T, S, CT, true> : k_vjp<NPE, T, S, CT, false>;
     FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
     int per_sm = 0;
-    FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, L.total));
+    FEM_CUDA(resident_blocks(&per_sm, f, 256, L.total));
     if (per_sm < 1) {
         set_error("backward kernel cannot be resident with %zu bytes of shared memory", L.total);
         return FEM_ERR_UNSUPPORTED;
@@ -907,7 +907,7 @@ __global__ void __launch_bounds__(256) k_vjp_sum(PlanView pv, const T *__restric
 
 static int grid_for(const void *f, int threads, size_t smem, int64_t np, const char *what, fem_status *st) {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem);
+    cudaError_t e = resident_blocks(&per_sm, f, threads, smem);
     if (e != cudaSuccess || per_sm < 1) {
         set_error("%s cannot be resident with %zu bytes of shared memory", what, smem);
         *st = e != cudaSuccess ? cuda_status(e, what) : FEM_ERR_UNSUPPORTED;
