@@ -116,3 +116,16 @@ def test_batched_and_backward(fem, kind, prec):
     b.pattern()
     for u, w in zip(a[2].vjp(X[2], c[2], G, prec), b.vjp(X[2], c[2], G, prec)):
         assert float((u - w).abs().max()) <= 4 * eps * float(w.abs().max())
+
+
+@pytest.mark.parametrize("kind", ["hex", "tet"])
+@pytest.mark.parametrize("opts", [{}, {"patch_entries": 40}, {"patch_entries": 900}],
+                         ids=lambda o: "-".join(f"{k}{v}" for k, v in o.items()) or "default")
+def test_load_vectors_equal_the_scatter(fem, kind, opts):
+    """The list form of the load vector (bricks) sums in the colour order too: equal bit for bit."""
+    for shape in SHAPES:
+        m = grid(kind, *shape)
+        a, b = pair(fem, m, **opts)
+        for prec, dt in (("mixed", torch.float32), ("mixed", torch.float64), ("fp64", torch.float64)):
+            X, c = dev(m.X, dt), dev(m.c, dt)
+            assert torch.equal(a.load_vector(X, c, prec), b.load_vector(X, c, prec))
