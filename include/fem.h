@@ -85,10 +85,12 @@ typedef struct {
                                     (brick 4, tetrahedron 10). */
     int valence_threshold;       /* mixed mode: entries with more contributions than
                                     this are summed in FP64.  Default 8. */
-    int patch_entries;           /* lower-CSR entries owned by one thread block (0 = default) */
+    int patch_entries;           /* lower-CSR entries owned by one thread block (0 = default; a
+                                    size of 3073 to 4096 is an upper bound: scalar operators
+                                    then take their default, which is smaller) */
     int block_threads;           /* threads per block of the patch kernels (0 = default) */
     int blocks_per_sm;           /* resident blocks per SM for the patch kernels (0 = default) */
-    int locality_order;          /* 1 = order nodes along a Morton curve of X (default); 0 = by id */
+    int locality_order;          /* 1 = order nodes along a Hilbert curve of X (default); 0 = by id */
     int fp64_sums;               /* mixed mode, high-valence entries: 0 (default) = error-free
                                     FP32 pair summation (TwoSum, accurate to ~2^-48 like an
                                     FP64 sum, rounded once); 1 = FP64 adds */
@@ -143,7 +145,7 @@ typedef struct {
                                     device staging and copied out in one transfer; n > 1 =
                                     the rows are split into n contiguous ranges of about
                                     n_nodes / n rows (the node order runs range by range,
-                                    each along its own Morton curve, and the node patches
+                                    each along its own Hilbert curve, and the node patches
                                     are planned inside the ranges; fixed at
                                     fem_mesh_create), and range k + 1 is built into one of two device
                                     slots while range k's values are copied to vals_host
@@ -204,7 +206,9 @@ typedef struct {
                                     tiles, closure_elems = n_elems, max_patch_entries = the
                                     largest tile's accumulator entries, max_patch_cnodes its
                                     rows) */
-    size_t live_bytes;           /* device bytes the library holds for the mesh now */
+    size_t live_bytes;           /* device bytes the library holds for the mesh now (without
+                                    a budget: whole slabs of up to 64 MB that its buffers
+                                    are carved from) */
     size_t peak_bytes;           /* the most it has held at once */
     int32_t n_chunks;            /* row ranges of the host pipeline (fem_options.host_chunks;
                                     1 = none) */

@@ -478,15 +478,6 @@ fem_status launch_order_x(const Plan &P, const float *X, float *xrank, cudaStrea
     return FEM_OK;
 }
 
-// Single meshes from this many nodes on have their FP32 coordinates put in locality
-// order first, so that the patches copy them in runs of 16-byte rows instead of three
-// 4-byte words a node at its id: 1M permuted bricks 175.7 -> 171.3 us with the extra
-// launch, 27M in natural numbering (whose ids come in runs by themselves) 3.84 -> 3.89
-// ms.  Below, the launch costs more than it saves (80,000 bricks' mass matrix and load
-// vector 43 us with it, 37 without).  Batches copy by id too (512 meshes: the extra
-// pass 0.13 ms).
-static constexpr int64_t XRANK_MIN = 1 << 18;
-
 GatherSmem gather_smem_layout(const GatherMax &g, int npe, bool fused, size_t accsize, size_t xsize, size_t csize) {
     GatherSmem L{};
     auto up = [](size_t v) { return (v + 15) & ~(size_t)15; };
@@ -543,7 +534,7 @@ static fem_status launch_gather_t(const PatchArgs &a, cudaStream_t s) {
     pv.val_off = a.val_off;
     const float *xr = nullptr;
     if constexpr (FUSED && sizeof(S) == 4) {
-        if (a.xrank && P.n_nodes >= XRANK_MIN) {
+        if (a.xrank) {
             xr = a.xrank;
             if (!a.x_ordered) FEM_TRY(launch_order_x(P, (const float *)a.X, a.xrank, s));
         }

@@ -98,6 +98,7 @@ struct Plan {
     DevBuf<int32_t> patch_acc, own_acc, own_row, node_patch, own_idx;
     DevBuf<uint8_t> own_hv;
     Closure full;          // closure of every patch, when it fits the memory budget
+    bool id_runs = false;  // neighbours in locality order often have consecutive ids
     bool chunked = false;  // closures built per patch group at each numeric call
     // aggregate statistics (over all groups when chunked)
     int64_t total_cnodes = 0, total_celems = 0, max_cnodes = 0, max_celems = 0;
@@ -146,6 +147,7 @@ struct Plan {
         n_patches = max_acc = max_own = total_cnodes = total_celems = max_cnodes = max_celems = 0;
         n_colors = 0;
         chunked = false;
+        id_runs = false;
         any_hv = false;
         chunk_row.clear();
         chunk_val.clear();

@@ -276,9 +276,9 @@ fem_status build_locality_order(fem_mesh m, const void *X, fem_dtype xd, cudaStr
     DevBuf<uint32_t> alt_vals;
     DevBuf<int64_t> hist, rows;
     FEM_TRY(bb.alloc(m->arena, 6 * (size_t)nr, "bbox"));
-    FEM_TRY(keys.alloc(m->arena, N, "morton keys"));
-    FEM_TRY(alt.alloc(m->arena, N, "morton keys'"));
-    FEM_TRY(alt_vals.alloc(m->arena, N, "morton vals'"));
+    FEM_TRY(keys.alloc(m->arena, N, "curve keys"));
+    FEM_TRY(alt.alloc(m->arena, N, "curve keys'"));
+    FEM_TRY(alt_vals.alloc(m->arena, N, "curve vals'"));
     FEM_TRY(hist.alloc(m->arena, radix_hist_elems(N), "radix histogram"));
     std::vector<unsigned long long> init(6 * (size_t)nr);
     for (int k = 0; k < nr; ++k)
@@ -343,12 +343,41 @@ __global__ void k_inc_sort(const int64_t *inc_ptr, int32_t *inc_elem, int64_t N)
     }
 }
 
+// Single meshes from this many nodes on have their FP32 coordinates put in locality
+// order first, so that the patches copy them in runs of 16-byte rows instead of three
+// 4-byte words a node at its id: 1M permuted bricks 175.7 -> 171.3 us with the extra
+// launch, the backward of 15.6M 6.84 -> 5.97 ms.  Below, the launch costs more than it
+// saves (80,000 bricks' mass matrix and load vector 43 us with it, 37 without).  Where
+// the ids come in runs by themselves (Plan::id_runs: natural numbering, a third of the
+// steps along the curve) it only costs: 27M bricks 3.84 -> 3.89 ms, the backward of
+// 15.6M 3.86 -> 3.99.  Batches copy by id too (512 meshes: the extra pass 0.13 ms).
+static constexpr int64_t XRANK_MIN = 1 << 18;
+
+// Steps of the node order that go to the next or the previous id.
+__global__ void k_id_runs(const int32_t *__restrict__ order, int64_t N, unsigned long long *steps) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    bool run = false;
+    if (i + 1 < N) {
+        const int32_t d = order[i + 1] - order[i];
+        run = d == 1 || d == -1;
+    }
+    const int n = __syncthreads_count(run);
+    if (threadIdx.x == 0 && n > 0) atomicAdd(steps, (unsigned long long)n);
+}
+
+// mx[0]: the largest incidence; with ISOLATED, mx[1]: 1 if a node has no element.
+template <bool ISOLATED>
 __global__ void k_max_deg(const int64_t *inc_ptr, int64_t N, unsigned long long *mx) {
-    unsigned long long m = 0;
-    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < N; g += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (unsigned long long)(inc_ptr[g + 1] - inc_ptr[g]));
+    unsigned long long m = 0, none = 0;
+    for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < N; g += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned long long d = (unsigned long long)(inc_ptr[g + 1] - inc_ptr[g]);
+        m = max(m, d);
+        if (d == 0) none = 1;
+    }
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(mx, m);
+    if constexpr (ISOLATED)
+        if (none) atomicMax(mx + 1, none);
 }
 
 // ------------------------------------------------------------- row pattern
@@ -1037,11 +1066,15 @@ fem_status build_pattern(fem_mesh m, cudaStream_t s) {
     unsigned long long max_deg = 0;
     {
         DevBuf<unsigned long long> mx;
-        FEM_TRY(mx.alloc(ar, 1, "max"));
-        FEM_CUDA(cudaMemsetAsync(mx.ptr, 0, sizeof(unsigned long long), s));
-        k_max_deg<<<grid_for(N), TPB, 0, s>>>(m->inc_ptr.ptr, N, mx.ptr);
+        unsigned long long h[2] = {0, 0};
+        FEM_TRY(mx.alloc(ar, 2, "max"));
+        FEM_CUDA(cudaMemsetAsync(mx.ptr, 0, sizeof(h), s));
+        k_max_deg<true><<<grid_for(N), TPB, 0, s>>>(m->inc_ptr.ptr, N, mx.ptr);
         FEM_LAUNCHED("k_max_deg");
-        FEM_TRY(read_scalar(mx.ptr, &max_deg, s));
+        FEM_CUDA(cudaMemcpyAsync(h, mx.ptr, sizeof(h), cudaMemcpyDeviceToHost, s));
+        FEM_CUDA(cudaStreamSynchronize(s));
+        max_deg = h[0];
+        if (h[1]) m->no_lists = true;  // gather lists hold a diagonal for every row
     }
     m->max_deg = (int64_t)max_deg;
     const int cap = (int)(max_deg * npe);
@@ -1561,9 +1594,10 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         const fem_status st = build_gather_lists(m, cl, s);
         if (st != FEM_OK && st != FEM_ERR_BUDGET) return st;
         if (cl.lists.ready) {
-            // coordinates in locality order, filled by each mixed build (refused by the
-            // budget: the builds gather them from X)
-            if (m->xrank.n < 4 * (size_t)m->n_nodes && m->xrank.alloc(ar, 4 * (size_t)m->n_nodes, "ordered X") != FEM_OK)
+            // coordinates in locality order, filled by each mixed call (refused by the
+            // budget: the kernels gather them from X)
+            if (m->n_nodes >= XRANK_MIN && !P.id_runs && m->xrank.n < 4 * (size_t)m->n_nodes &&
+                m->xrank.alloc(ar, 4 * (size_t)m->n_nodes, "ordered X") != FEM_OK)
                 cudaGetLastError();
             return FEM_OK;
         }
@@ -1665,6 +1699,11 @@ static fem_status plan_groups(fem_mesh m, cudaStream_t s) {
     });
 }
 
+// Whether patches for gather lists take the size that suits them (build_plan_cap).
+static bool default_list_patches(fem_mesh m) {
+    return m->opt.patch_entries <= 0 || (m->opt.patch_entries > 3072 && m->opt.patch_entries <= 4096);
+}
+
 // Global part of the plan (patches of consecutive nodes in locality order, the
 // owned-row tables), then the closures of all patches at once if the memory
 // budget holds them, else closures are built per patch group by each numeric call.
@@ -1682,12 +1721,16 @@ static fem_status build_plan_cap(fem_mesh m, cudaStream_t s, int64_t cap_in) {
     // 171 us at 3,072 entries, 180 at 2,688, 199 at 4,096 with one block an SM).
     // Meshes of up to 2^18 nodes take fewer: their odd shapes have larger closures, and
     // a batch's launch is sized by the largest of all (512 meshes: 2.71 ms at 2,816,
-    // 3.31 at 3,072).  Tetrahedra: 152 us at 1,024, 173 at 1,280 (3.07M).
+    // 3.31 at 3,072).  Tetrahedra: 152 us at 1,024, 173 at 1,280 (3.07M).  A size given
+    // between 3,072 and 4,096 (the smallest the tuner tries) is a bound that the default
+    // stays within; from about 5,000 the lists no longer fit and the scatter runs.
     int64_t cap_entries = cap_in > 0 ? cap_in : m->opt.patch_entries;
-    if (cap_entries <= 0) {
-        if (elastic) cap_entries = m->npe == 8 ? 4096 : 1536;
-        else if (!wants_lists(m)) cap_entries = 8192;
-        else cap_entries = m->npe == 4 ? 1024 : N < (1 << 18) ? 2816 : 3072;
+    if (elastic) {
+        if (cap_entries <= 0) cap_entries = m->npe == 8 ? 4096 : 1536;
+    } else if (!wants_lists(m)) {
+        if (cap_entries <= 0) cap_entries = 8192;
+    } else if (cap_in <= 0 && default_list_patches(m)) {
+        cap_entries = m->npe == 4 ? 1024 : N < (1 << 18) ? 2816 : 3072;
     }
     if (cap_entries < 2 * (int64_t)m->max_row_len) cap_entries = 2 * (int64_t)m->max_row_len;
     P.cap_entries = cap_entries;
@@ -1790,12 +1833,23 @@ static fem_status build_plan_cap(fem_mesh m, cudaStream_t s, int64_t cap_in) {
     FEM_LAUNCHED("k_patch_nodes");
     k_patch_acc<<<grid_for(npatch), TPB, 0, s>>>(pre.ptr, P.patch_node_ptr.ptr, npatch, P.patch_acc.ptr);
     FEM_LAUNCHED("k_patch_acc");
+    unsigned long long id_steps = 0;
+    DevBuf<unsigned long long> steps;
+    if (wants_lists(m) && N >= XRANK_MIN) {
+        FEM_TRY(steps.alloc(ar, 1, "id steps"));
+        FEM_CUDA(cudaMemsetAsync(steps.ptr, 0, sizeof(unsigned long long), s));
+        k_id_runs<<<(unsigned)cdiv(N, TPB), TPB, 0, s>>>(m->order.ptr, N, steps.ptr);
+        FEM_LAUNCHED("k_id_runs");
+        FEM_CUDA(cudaMemcpyAsync(&id_steps, steps.ptr, sizeof(id_steps), cudaMemcpyDeviceToHost, s));
+    }
     std::vector<int64_t> h_pn(npatch + 1);
     std::vector<int32_t> h_acc(npatch);
     FEM_CUDA(cudaMemcpyAsync(h_pn.data(), P.patch_node_ptr.ptr, (npatch + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
     FEM_CUDA(cudaMemcpyAsync(h_acc.data(), P.patch_acc.ptr, npatch * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     FEM_CUDA(cudaStreamSynchronize(s));
     pre.free();
+    steps.free();
+    P.id_runs = id_steps > (unsigned long long)N / 8;
     for (int64_t p = 0; p < npatch; ++p) {
         P.max_own = std::max(P.max_own, h_pn[p + 1] - h_pn[p]);
         P.max_acc = std::max(P.max_acc, (int64_t)h_acc[p]);
@@ -1835,7 +1889,18 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
     FEM_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     int64_t cap = 0;
     for (;;) {
-        FEM_TRY(build_plan_cap(m, s, cap));
+        const fem_status st = build_plan_cap(m, s, cap);
+        // Patches of a size chosen for the gather lists, but no lists (the budget refuses
+        // them, or a closure is out of their range): planned again at the scatter's size
+        // (27M bricks in the patch groups of a 7 GB budget: 57 ms a build at the lists'
+        // size, 51 at the scatter's).
+        if (cap == 0 && (st == FEM_OK || st == FEM_ERR_BUDGET) && wants_lists(m) && !m->plan.full.lists.ready &&
+            default_list_patches(m)) {
+            cudaGetLastError();
+            m->no_lists = true;
+            continue;
+        }
+        FEM_TRY(st);
         if (m->opt.operator_kind == 2) return FEM_OK;
         PlanMax pm;
         pm.add(m->plan);
@@ -1877,7 +1942,7 @@ fem_status pattern_steps_incidence(const int32_t *E, int64_t nel, int npe, int64
     FEM_LAUNCHED("k_inc_fill");
     k_inc_sort<<<grid_for(N), TPB, 0, s>>>(inc_ptr, inc_elem, N);
     FEM_LAUNCHED("k_inc_sort");
-    k_max_deg<<<grid_for(N), TPB, 0, s>>>(inc_ptr, N, mx);
+    k_max_deg<false><<<grid_for(N), TPB, 0, s>>>(inc_ptr, N, mx);
     FEM_LAUNCHED("k_max_deg");
     return FEM_OK;
 }

@@ -129,3 +129,29 @@ def test_load_vectors_equal_the_scatter(fem, kind, opts):
         for prec, dt in (("mixed", torch.float32), ("mixed", torch.float64), ("fp64", torch.float64)):
             X, c = dev(m.X, dt), dev(m.c, dt)
             assert torch.equal(a.load_vector(X, c, prec), b.load_vector(X, c, prec))
+
+
+@pytest.mark.parametrize("kind", ["hex", "tet"])
+def test_patch_sizes_follow_the_route(fem, kind):
+    """Lists and scatter have default patch sizes of their own: a mesh that cannot have
+    lists is planned at the scatter's, and 4,096 entries bound the lists' default."""
+    m = grid(kind, *((40, 40, 40) if kind == "hex" else (24, 24, 24)))
+    E, X = dev(m.E, torch.int32), dev(m.X, torch.float64)
+    c = dev(m.c, torch.float32)
+
+    def planned(n=m.n_nodes, x=X, **opts):
+        mesh = fem.Mesh(E, n, X=x, **opts)
+        v = mesh.build_K(x.float(), c, "mixed")
+        return mesh.info(), v
+
+    lists, scatter = planned(), planned(fp64_fused=1)
+    assert lists[0]["n_patches"] > scatter[0]["n_patches"]
+    bound = planned(patch_entries=4096)
+    assert bound[0]["n_patches"] == lists[0]["n_patches"] and torch.equal(bound[1], lists[1])
+    far = torch.cat([X, X[:1]])  # one node of no element
+    lone, other = planned(m.n_nodes + 1, far), planned(m.n_nodes + 1, far, fp64_fused=1)
+    assert lone[0]["n_patches"] == other[0]["n_patches"] and torch.equal(lone[1], other[1])
+    budget = int(0.7 * scatter[0]["plan_bytes"])
+    tight, same = planned(mem_budget_bytes=budget), planned(mem_budget_bytes=budget, fp64_fused=1)
+    assert tight[0]["n_groups"] == same[0]["n_groups"] and tight[0]["n_patches"] == same[0]["n_patches"]
+    assert torch.equal(tight[1], same[1])
