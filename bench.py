@@ -151,8 +151,8 @@ def measured_peaks():
 
 
 # the sources that determine the patch kernel's code and its plan's layout
-KERNEL_SOURCES = ("element.cuh", "elem_ops.cuh", "mesh.cuh", "tile.cuh", "numeric.cu", "numeric.cuh", "phases.cuh",
-                  "symbolic.cu", "tile.cu", "tile_plan.cu")
+KERNEL_SOURCES = ("element.cuh", "elem_ops.cuh", "gather.cu", "gather.cuh", "gather_plan.cu", "mesh.cuh", "numeric.cu",
+                  "numeric.cuh", "pair.cuh", "phases.cuh", "symbolic.cu", "tile.cu", "tile.cuh", "tile_plan.cu")
 
 
 def source_hash():
@@ -184,7 +184,8 @@ def algorithmic_bytes(n_nodes, n_elems, npe, nnz, xsize, csize, vsize):
 # 12 edge vectors (36), Jacobian rows at the 8 points (216), per point cofactor
 # rows, determinant, reciprocal, 6 Gram entries scaled (8 x 73 = 584), distortion
 # test (17), axis sums (12), 3 diagonal-direction tables (120), 3 cross tables
-# (300), 36 packed entries of 9 terms scaled by c/8 (648).
+# (300), 36 packed entries of 9 terms scaled by c/8 (648).  A nominal count: the
+# kernels share sums between the packed entries and do fewer.
 BRICK_FLOPS = 36 + 216 + 584 + 17 + 12 + 120 + 300 + 648
 SMS, FP32_LANES = 152, 128
 
@@ -451,7 +452,9 @@ def run_ours(args):
     alg = algorithmic_bytes(m.n_nodes, m.n_elems, 8, nnz, 4, 4, 4)
     alg64 = algorithmic_bytes(m.n_nodes, m.n_elems, 8, nnz, 8, 8, 8)
     achieved = alg / (ms_step / 1e3) / 1e9
-    kernel = "k_tile" if info["assembly"] == 1 else "k_patch"
+    # patches of up to 4,096 entries run on gather lists, larger ones on the colour-ordered scatter
+    lists = tuning.get("patch_entries", 0) <= 4096
+    kernel = "k_tile" if info["assembly"] == 1 else "k_gather" if lists else "k_patch"
     wkey = f"hex8_n{args.n}_mixed_{'t' if info['assembly'] == 1 else 'p'}{tuning.get('patch_entries', 0)}"
     sm_mhz = (clocks or {}).get("sm_mhz") or 2070.0
     alu_peak = SMS * FP32_LANES * 2 * sm_mhz * 1e6 / 1e12          # TFLOP/s at the sampled clock
@@ -459,7 +462,7 @@ def run_ours(args):
     roof = {"bound": "alu", "achieved": alu_achieved, "peak": alu_peak, "unit": "TFLOP/s",
             "frac": alu_achieved / alu_peak, "traffic": profiled_traffic(kernel, wkey),
             "peak_source": f"derived: {SMS} SMs x {FP32_LANES} FP32 lanes x 2 FLOP x {sm_mhz:.0f} MHz (sampled)",
-            "kernel": f"{kernel} (fused integrate + assemble; bricks run its prefetching form k_patch_prefetch) and its launches",
+            "kernel": f"{kernel} (fused integrate + assemble) and its launches",
             "flops_per_element": BRICK_FLOPS,
             "hbm": {"achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "peak_source": f"{peak_kind} (MEASURED_PEAKS hbm_gbs)" if peak_kind == "measured" else peak_kind,
