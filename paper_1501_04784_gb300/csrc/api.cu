@@ -358,7 +358,6 @@ static PatchArgs patch_args(fem_mesh m, fem_prec p, bool fused) {
     if (!fused && m->opt.block_threads <= 0 && m->plan.full.lists.ready) a.threads = 512;
     if (is_elastic(m)) a.threads = elastic_threads(m->npe, m->opt.block_threads);  // its own default and cap
     a.blocks_per_sm = m->opt.blocks_per_sm;
-    if (fused && a.mixed && m->xrank.n >= 4 * (size_t)m->n_nodes) a.xrank = m->xrank.ptr;
     a.mode = kernel_mode(m->opt);
     a.wait = wait_ctl(m);
     return a;
@@ -501,6 +500,8 @@ fem_status fem_build_K(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype,
         if (st != FEM_ERR_BUDGET) return st;
     }
     PatchArgs a = patch_args(m, p, true);
+    const XrankUse ordered(m, a.mixed, x_dtype, s);
+    a.xrank = ordered.ptr();
     a.xd = x_dtype;
     a.cd = c_dtype;
     a.X = X;
@@ -564,6 +565,8 @@ static fem_status chunk_pipeline(fem_mesh m, fem_prec p, const void *X, fem_dtyp
         }
     }
     PatchArgs a = patch_args(m, p, !staged);
+    const XrankUse ordered(m, a.mixed && !staged, xd, s);  // over all the ranges
+    a.xrank = ordered.ptr();
     if (staged) {
         a.xd = a.cd = FEM_F64;
         a.ke = m->ke64.ptr;

@@ -478,6 +478,27 @@ fem_status launch_order_x(const Plan &P, const float *X, float *xrank, cudaStrea
     return FEM_OK;
 }
 
+XrankUse::XrankUse(fem_mesh m, bool mixed, fem_dtype xd, cudaStream_t s) : m_(m), s_(s) {
+    if (!mixed || xd != FEM_F32 || !m->plan.full.lists.ready || m->xrank.n < 4 * (size_t)m->n_nodes) return;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return;
+    }
+    lock_ = std::unique_lock<std::mutex>(m->xrank_mu);
+    if ((m->xrank_read || cudaEventCreateWithFlags(&m->xrank_read, cudaEventDisableTiming) == cudaSuccess) &&
+        cudaStreamWaitEvent(s, m->xrank_read, 0) == cudaSuccess) {
+        ptr_ = m->xrank.ptr;
+    } else {
+        cudaGetLastError();
+        lock_.unlock();
+    }
+}
+
+XrankUse::~XrankUse() {
+    if (ptr_ && cudaEventRecord(m_->xrank_read, s_) != cudaSuccess) cudaStreamSynchronize(s_);
+}
+
 GatherSmem gather_smem_layout(const GatherMax &g, int npe, bool fused, size_t accsize, size_t xsize, size_t csize) {
     GatherSmem L{};
     auto up = [](size_t v) { return (v + 15) & ~(size_t)15; };

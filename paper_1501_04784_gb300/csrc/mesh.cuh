@@ -14,6 +14,7 @@
 #include <cstring>
 #include <functional>
 #include <utility>
+#include <mutex>
 #include <vector>
 
 #include "common.cuh"
@@ -253,6 +254,7 @@ struct fem_mesh_s {
         for (cudaEvent_t e : stage_free)
             if (e) cudaEventDestroy(e);
         if (built) cudaEventDestroy(built);
+        if (xrank_read) cudaEventDestroy(xrank_read);
         for (int j = 0; j < 2; ++j) {
             if (chunk_built[j]) cudaEventDestroy(chunk_built[j]);
             if (slot_free[j]) cudaEventDestroy(slot_free[j]);
@@ -263,7 +265,11 @@ struct fem_mesh_s {
     // pipe is the bound there, so integrating each element once beats recomputing
     // it in every closure that contains it)
     fem::DevBuf<double> ke64;
-    fem::DevBuf<float> xrank;  // [n_nodes][4] FP32 coordinates in locality order (gather builds)
+    // [n_nodes][4] FP32 coordinates in locality order (gather builds): filled and read by
+    // one call at a time, see XrankUse
+    fem::DevBuf<float> xrank;
+    std::mutex xrank_mu;
+    cudaEvent_t xrank_read = nullptr;
     // host pipeline over row ranges: two device value slots used in turn, the
     // stream their copies to the host run on, chunk_built[j] recorded after the
     // build of the range in slot j, slot_free[j] after its copy out
@@ -298,6 +304,27 @@ bool wants_lists(fem_mesh m);
 // The full closure's accumulator targets (the colour-ordered scatter): plans mesh m
 // again without gather lists when the builds ran on those.
 fem_status ensure_targets(fem_mesh m, cudaStream_t s);
+// One call's use of the mesh's ordered coordinates.  A mixed build writes nothing of the
+// mesh's but its status word, and calls on several streams or threads rely on that, so
+// the buffer passes from call to call: a call's stream waits for the last reader's event,
+// and the host lock is held until this call's own event is recorded.  Null (the kernels
+// take X by node id, the same values) where the plan has no such buffer, and under
+// capture, as graphs replayed side by side would share it.  The wait and the record cost
+// the host about 1 us of a call.
+class XrankUse {
+  public:
+    XrankUse(fem_mesh m, bool mixed, fem_dtype xd, cudaStream_t s);
+    ~XrankUse();
+    XrankUse(const XrankUse &) = delete;
+    XrankUse &operator=(const XrankUse &) = delete;
+    float *ptr() const { return ptr_; }
+
+  private:
+    fem_mesh m_;
+    cudaStream_t s_;
+    std::unique_lock<std::mutex> lock_;
+    float *ptr_ = nullptr;
+};
 // Runs fn over the closure of every patch group (one group covering all patches
 // unless the plan is chunked under the memory budget).
 fem_status for_each_group(fem_mesh m, cudaStream_t s, const std::function<fem_status(const Closure &)> &fn);

@@ -974,13 +974,10 @@ static fem_status launch_vjp_elem_t(fem_mesh m, const Closure &cl, const void *X
         if (cl.lists.ready && (P.id_runs || m->nnz * (int64_t)sizeof(T) <= (128 << 20))) nt = 128;
     const int grid = grid_for((const void *)f, nt, L.total, np, "backward element kernel", &st);
     if (st != FEM_OK) return st;
-    const float4 *xr = nullptr;
-    if constexpr (sizeof(S) == 4) {
-        if (cl.lists.ready && m->xrank.n >= 4 * (size_t)m->n_nodes) {
-            FEM_TRY(launch_order_x(P, (const float *)X, m->xrank.ptr, s));
-            xr = reinterpret_cast<const float4 *>(m->xrank.ptr);
-        }
-    }
+    const XrankUse ordered(m, sizeof(T) == 4, sizeof(S) == 4 ? FEM_F32 : FEM_F64, s);
+    const float4 *xr = reinterpret_cast<const float4 *>(ordered.ptr());
+    if constexpr (sizeof(S) == 4)
+        if (xr) FEM_TRY(launch_order_x(P, (const float *)X, ordered.ptr(), s));
     f<<<grid, nt, L.total, s>>>(P.view(cl), m->rowptr.ptr, (const S *)X, xr, (const CT *)c, (const T *)G, (T *)dxe,
                                 (T *)dc, L, m->status.ptr);
     FEM_LAUNCHED("k_vjp_elem");
