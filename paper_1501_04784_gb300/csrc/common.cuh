@@ -150,6 +150,17 @@ inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 int num_sms();
 
+// Lets a kernel be launched with `bytes` of dynamic shared memory.  The limit belongs to
+// the kernel, not to a launch: set to each launch's own size, it can be lowered by another
+// mesh or thread between a launch's setting and the launch, or between a batch's tuning
+// and its capture.  So it is only ever raised (and set anew each time, in case the
+// device was reset).
+cudaError_t allow_smem_of(const void *kernel, size_t bytes);
+template <typename F>
+cudaError_t allow_smem(F kernel, size_t bytes) {
+    return allow_smem_of(reinterpret_cast<const void *>(kernel), bytes);
+}
+
 // cudaOccupancyMaxActiveBlocksPerMultiprocessor with its answers remembered: they depend
 // on the kernel, the device and the launch shape alone, and the query costs some 4 us
 // of every launch.  At most a few hundred shapes are kept.

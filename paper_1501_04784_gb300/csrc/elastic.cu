@@ -27,7 +27,7 @@ static constexpr int EL_INT_THREADS = 128;
 
 template <typename F>
 static fem_status el_set_smem(F *f, size_t bytes) {
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    FEM_CUDA(allow_smem(f, bytes));
     return FEM_OK;
 }
 

@@ -526,7 +526,7 @@ static fem_status launch_elastic_vjp_t(fem_mesh m, const Closure &cl, const void
                            : (size_t)P.max_own * 3 * sizeof(T)));
     L.total = o;
     auto f = staged ? k_elastic_vjp_elem<NPE, T, S, CT> : k_elastic_vjp<NPE, T, S, CT>;
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     int per_sm = 0;
     FEM_CUDA(resident_blocks(&per_sm, f, 256, L.total));
     if (per_sm < 1) {

@@ -527,7 +527,7 @@ GatherSmem gather_smem_layout(const GatherMax &g, int npe, bool fused, size_t ac
 // Resident blocks of f at `threads` threads and L bytes, opted in; 0 if none fits.
 template <typename F>
 static fem_status resident(F *f, int threads, size_t bytes, int *per_sm) {
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    FEM_CUDA(allow_smem(f, bytes));
     FEM_CUDA(resident_blocks(per_sm, f, threads, bytes));
     if (*per_sm < 1) {
         set_error("the gather kernel cannot be resident with %d threads and %zu bytes of shared memory", threads, bytes);

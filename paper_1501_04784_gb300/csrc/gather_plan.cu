@@ -345,7 +345,7 @@ fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s) {
     int top_step = 1;  // the largest power of two below the longest row's length
     while (2 * top_step < m->max_row_len) top_step *= 2;
     auto f = m->npe == 8 ? k_gather_lists<8> : k_gather_lists<4>;
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     for (int pass = 0; pass < 2; ++pass) {
         FEM_TRY(G.words.alloc(m->arena, cap, "gather lists"));
         FEM_CUDA(cudaMemsetAsync(cursor.ptr, 0, 2 * sizeof(unsigned long long), s));

@@ -217,7 +217,7 @@ static fem_status launch_load_t(fem_mesh m, const Closure &cl, const void *X, co
             L.fe = al16((size_t)P.max_cnodes * 3 * sizeof(S));
             L.total = al16(L.fe + (size_t)P.max_celems * NPE * sizeof(T));
             auto f = k_load_lists<NPE, T, S, CT, MIXED>;
-            FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+            FEM_CUDA(allow_smem(f, L.total));
             int per_sm = 0;
             FEM_CUDA(resident_blocks(&per_sm, f, 256, L.total));
             const int64_t np = cl.p1 - cl.p0;
@@ -239,7 +239,7 @@ static fem_status launch_load_t(fem_mesh m, const Closure &cl, const void *X, co
     o = al16(o + (size_t)NC * P.max_own * sizeof(T));
     L.total = o;
     auto f = k_load<NPE, T, S, CT, MIXED, NC>;
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     int per_sm = 0;
     FEM_CUDA(resident_blocks(&per_sm, f, 256, L.total));
     if (per_sm < 1) {

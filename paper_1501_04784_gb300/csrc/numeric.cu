@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(patch_max_threads(NPE), patch_min_blocks(NPE))
 // ------------------------------------------------------------------ launchers
 template <typename F>
 static fem_status set_smem(F *f, size_t bytes) {
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    FEM_CUDA(allow_smem(f, bytes));
     return FEM_OK;
 }
 

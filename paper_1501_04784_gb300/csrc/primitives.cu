@@ -1,5 +1,6 @@
 // primitives.cu -- status plumbing, budgeted allocation, and the device-wide
 // scan and radix sort used by the symbolic phase.
+#include <algorithm>
 #include <cstdarg>
 #include <cstring>
 #include <iterator>
@@ -24,6 +25,7 @@ void set_error(const char *fmt, ...) {
 
 fem_status cuda_status(cudaError_t e, const char *what) {
     set_error("%s: %s", what, cudaGetErrorString(e));
+    cudaGetLastError();  // reported here, not by the next call that asks after its launches
     return e == cudaErrorMemoryAllocation ? FEM_ERR_OOM : FEM_ERR_CUDA;
 }
 
@@ -172,6 +174,20 @@ bool Arena::uncarve(void *p, size_t size) {
         return true;
     }
     return false;
+}
+
+cudaError_t allow_smem_of(const void *kernel, size_t bytes) {
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, size_t> largest;  // one entry a kernel and device
+    int dev = 0;
+    const cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    size_t &top = largest[{kernel, dev}];
+    const size_t want = std::max(top, bytes);
+    const cudaError_t st = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)want);
+    if (st == cudaSuccess) top = want;
+    return st;
 }
 
 cudaError_t resident_blocks_of(int *n, const void *kernel, int threads, size_t smem) {

@@ -993,8 +993,8 @@ static fem_status launch_row_pattern(const int32_t *E, int npe, int64_t N, const
 #undef FEM_RP
     const size_t smem = (size_t)wpb * (cap > 0 ? cap : 1) * sizeof(int32_t);
     if (smem > (48u << 10)) {
-        if (npe == 8) FEM_CUDA(cudaFuncSetAttribute(k_row_pattern<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        else FEM_CUDA(cudaFuncSetAttribute(k_row_pattern<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        if (npe == 8) FEM_CUDA(allow_smem(k_row_pattern<8>, smem));
+        else FEM_CUDA(allow_smem(k_row_pattern<4>, smem));
     }
     if (npe == 8) k_row_pattern<8><<<grid, wpb * 32, smem, s>>>(E, inc_ptr, inc_elem, N, cap, cnt, rowptr, col);
     else k_row_pattern<4><<<grid, wpb * 32, smem, s>>>(E, inc_ptr, inc_elem, N, cap, cnt, rowptr, col);
@@ -1353,7 +1353,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         FEM_CUDA(cudaMemsetAsync(ovf.ptr, 0, sizeof(int), s));
         const size_t smem = 2 * (size_t)hsize * sizeof(uint32_t);
         auto f = npe == 8 ? k_patch_celems<8> : k_patch_celems<4>;
-        FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        FEM_CUDA(allow_smem(f, smem));
         int per_sm = 1;
         FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, smem));
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np_, (int64_t)num_sms() * std::max(per_sm, 1)));
@@ -1445,11 +1445,11 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         // shared memory small)
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np_, (int64_t)num_sms() * 16));
         if (npe == 8) {
-            FEM_CUDA(cudaFuncSetAttribute(k_color<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            FEM_CUDA(allow_smem(k_color<8>, smem));
             k_color<8><<<grid, 128, smem, s>>>(ckeys.ptr, cl.patch_elem_ptr.ptr, P.patch_node_ptr.ptr + p0, m->E,
                                                P.node_patch.ptr, P.own_idx.ptr, np_, p0, color.ptr, mxc.ptr);
         } else {
-            FEM_CUDA(cudaFuncSetAttribute(k_color<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            FEM_CUDA(allow_smem(k_color<4>, smem));
             k_color<4><<<grid, 128, smem, s>>>(ckeys.ptr, cl.patch_elem_ptr.ptr, P.patch_node_ptr.ptr + p0, m->E,
                                                P.node_patch.ptr, P.own_idx.ptr, np_, p0, color.ptr, mxc.ptr);
         }
@@ -1467,7 +1467,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         if (cl.max_celems <= SET_MAX_SLOTS / 2) {
             // per patch in shared memory
             const size_t csm = (size_t)pow2_at_least((int)std::max<int64_t>(cl.max_celems, 1)) * sizeof(uint64_t);
-            FEM_CUDA(cudaFuncSetAttribute(k_patch_color_order, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm));
+            FEM_CUDA(allow_smem(k_patch_color_order, csm));
             const unsigned cgrid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np_, (int64_t)num_sms() * 2));
             k_patch_color_order<<<cgrid, 512, csm, s>>>(ckeys.ptr, color.ptr, cl.patch_elem_ptr.ptr, np_, ck2.ptr);
             FEM_LAUNCHED("k_patch_color_order");
@@ -1515,7 +1515,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         FEM_CUDA(cudaMemsetAsync(ovf.ptr, 0, sizeof(int), s));
         const size_t smem = 2 * (size_t)hsize * sizeof(uint32_t);
         auto f = npe == 8 ? k_patch_cnodes<8> : k_patch_cnodes<4>;
-        FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        FEM_CUDA(allow_smem(f, smem));
         int per_sm = 1;
         FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, 256, smem));
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np_, (int64_t)num_sms() * std::max(per_sm, 1)));
@@ -1579,7 +1579,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         const size_t smem = (size_t)std::max<int64_t>(cl.max_cnodes, 1) * sizeof(int32_t);
         const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np_, (int64_t)num_sms() * 8));
         auto f = npe == 8 ? k_celem_fill<8> : k_celem_fill<4>;
-        FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        FEM_CUDA(allow_smem(f, smem));
         f<<<grid, TPB, smem, s>>>(ckeys.ptr, np_, m->E, cnkeys.ptr, cl.patch_cnode_ptr.ptr, m->rowptr.ptr, m->col.ptr,
                                   P.pos_stride, ot, cl.celem_id.ptr, cl.celem_color.ptr, cl.celem_lnode.ptr,
                                   with_pos ? cl.celem_pos.ptr : nullptr,

@@ -469,7 +469,7 @@ static fem_status tile_batched_config_t(const TileMax &tm, int threads, int bloc
         set_error("a tile of the batch needs %zu bytes of shared memory (limit %d)", L.total, max_optin);
         return FEM_ERR_UNSUPPORTED;
     }
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     int per_sm = 0;
     FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, L.total));
     if (per_sm < 1) {
@@ -543,7 +543,7 @@ static fem_status launch_tile_t(const TileArgs &a, cudaStream_t s) {
         set_error("an element tile needs %zu bytes of shared memory (limit %d); lower tile_elems", L.total, max_optin);
         return FEM_ERR_UNSUPPORTED;
     }
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     int per_sm = 0;
     FEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, a.threads, L.total));
     if (per_sm < 1) {

@@ -455,8 +455,8 @@ fem_status build_tiles(fem_mesh m, cudaStream_t s) {
     FEM_CUDA(cudaGetDevice(&dev));
     FEM_CUDA(cudaDeviceGetAttribute(&max_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     const size_t count_smem = (size_t)TP_MAX_KEYS * 4;
-    if (npe == 8) FEM_CUDA(cudaFuncSetAttribute(k_tile_count<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)count_smem));
-    else FEM_CUDA(cudaFuncSetAttribute(k_tile_count<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)count_smem));
+    if (npe == 8) FEM_CUDA(allow_smem(k_tile_count<8>, count_smem));
+    else FEM_CUDA(allow_smem(k_tile_count<4>, count_smem));
     DevBuf<int64_t> tep, ncn, nacc, nbord;
     std::vector<int64_t> h_tep, h_ncn, h_nacc, h_nbord;
     int64_t nt = 0, max_ncn = 0, max_acc = 0, pmax = 0;
@@ -586,10 +586,10 @@ fem_status build_tiles(fem_mesh m, cudaStream_t s) {
         const FillSmem L = fill_layout(npe, pmax, max_ncn);
         const unsigned grid = (unsigned)std::min<int64_t>(nt, (int64_t)num_sms() * 4);
         if (npe == 8) {
-            FEM_CUDA(cudaFuncSetAttribute(k_tile_fill<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+            FEM_CUDA(allow_smem(k_tile_fill<8>, L.total));
             k_tile_fill<8><<<grid, TP_THREADS, L.total, s>>>(in, nt, out, L);
         } else {
-            FEM_CUDA(cudaFuncSetAttribute(k_tile_fill<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+            FEM_CUDA(allow_smem(k_tile_fill<4>, L.total));
             k_tile_fill<4><<<grid, TP_THREADS, L.total, s>>>(in, nt, out, L);
         }
         FEM_LAUNCHED("k_tile_fill");

@@ -532,7 +532,7 @@ static fem_status launch_vjp_t(fem_mesh m, const Closure &cl, const void *X, con
     o = a16(o + (size_t)P.max_own * 3 * sizeof(T));
     L.total = o;
     auto f = m->opt.operator_kind == 1 ? k_vjp<NPE, T, S, CT, true> : k_vjp<NPE, T, S, CT, false>;
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     int per_sm = 0;
     FEM_CUDA(resident_blocks(&per_sm, f, 256, L.total));
     if (per_sm < 1) {
@@ -939,7 +939,7 @@ static fem_status launch_vjp_sum_t(fem_mesh m, const Closure &cl, const void *dx
     L.out = a16((size_t)m->plan.max_celems * NPE * 3 * sizeof(T));
     L.total = a16(L.out + (size_t)m->plan.max_own * 3 * sizeof(T));
     auto f = k_vjp_sum<NPE, T>;
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     fem_status st;
     const int grid = grid_for((const void *)f, 256, L.total, cl.p1 - cl.p0, "backward sum kernel", &st);
     if (st != FEM_OK) return st;
@@ -954,7 +954,7 @@ static fem_status launch_vjp_elem_t(fem_mesh m, const Closure &cl, const void *X
     const Plan &P = m->plan;
     const ElemSmem L = elem_smem(P, cl, sizeof(S));
     auto f = m->opt.operator_kind == 1 ? k_vjp_elem<NPE, T, S, CT, true> : k_vjp_elem<NPE, T, S, CT, false>;
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     if constexpr (NPE == 4) {
         // tets: shared memory for two blocks per SM, the rest of the unified L1/shared
         // array kept as L1 for the element's gathers
@@ -997,7 +997,7 @@ static fem_status launch_gather_t(fem_mesh m, const Closure &cl, const void *dxe
     o = a16(o + (size_t)P.max_own * 3 * sizeof(T));
     L.total = o;
     auto f = k_vjp_gather<NPE, T>;
-    FEM_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.total));
+    FEM_CUDA(allow_smem(f, L.total));
     const int64_t np = cl.p1 - cl.p0;
     if (np <= 0) return FEM_OK;
     fem_status st;
