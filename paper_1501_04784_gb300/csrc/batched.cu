@@ -10,6 +10,12 @@
 // (the tuner), and captures the single launch into a CUDA graph.  Later calls
 // with the same meshes only refresh the descriptor table (inputs and outputs may
 // move) and replay the graph: one copy and one graph launch per build.
+//
+// A batch that no one launch can build is cut into parts, a launch each in the same
+// graph: meshes with gather lists and meshes planned for the scatter run different
+// kernels, and a gather launch's shared memory is sized by the largest closure, node
+// list and row count of all its meshes, which may come from three of them and not fit
+// together.
 #include <algorithm>
 #include <memory>
 #include <mutex>
@@ -20,6 +26,15 @@
 
 namespace fem {
 
+// The meshes of one launch: places [first, first + n) of the context's tables.
+struct BatchPart {
+    bool gather = false;   // every mesh has gather lists, and the launch runs on them
+    int first = 0, n = 0;
+    GatherMax gm;          // largest patch sizes of its meshes (gather)
+    GatherPatch *d_gpatch = nullptr;
+    BatchLaunch bl;
+};
+
 struct BatchCtx {
     std::vector<fem_mesh> meshes;
     bool mixed = true;
@@ -27,24 +42,22 @@ struct BatchCtx {
     int npe = 8;
     bool elastic = false;  // the elasticity operator (operator_kind 2)
     bool tiles = false;    // the meshes build on element tiles
-    bool gather = false;   // every mesh has gather lists
-    GatherPatch *d_gpatch = nullptr;
+    std::vector<BatchPart> parts;
+    std::vector<int> place, mesh_at;  // place of mesh i in the tables, and the other way round
     BatchItem *d_items = nullptr;
     TileBatchItem *d_titems = nullptr;
     std::vector<TileBatchItem> h_titems;
     int64_t *d_prefix = nullptr;
     int64_t *d_bprefix = nullptr;  // tiles: prefix sums of the border rows
     std::vector<BatchItem> h_items;
-    BatchLaunch bl;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    float tuned_ms = 0.f;
-    int tried = 0;
     ~BatchCtx() {
         if (exec) cudaGraphExecDestroy(exec);
         if (graph) cudaGraphDestroy(graph);
         if (d_items) cudaFree(d_items);
-        if (d_gpatch) cudaFree(d_gpatch);
+        for (BatchPart &q : parts)
+            if (q.d_gpatch) cudaFree(q.d_gpatch);
         if (d_titems) cudaFree(d_titems);
         if (d_prefix) cudaFree(d_prefix);
         if (d_bprefix) cudaFree(d_bprefix);
@@ -74,16 +87,16 @@ static void fill_items(BatchCtx &c, const void *const *X, const void *const *cc,
     if (c.tiles) {
         for (size_t i = 0; i < c.meshes.size(); ++i) {
             const fem_mesh m = c.meshes[i];
-            c.h_titems[i] = TileBatchItem{m->tiles.view(m), X[i], cc[i], vals[i], m->tiles.partial.ptr,
+            c.h_titems[c.place[i]] = TileBatchItem{m->tiles.view(m), X[i], cc[i], vals[i], m->tiles.partial.ptr,
                                           mesh_threshold(m), 0};
         }
         return;
     }
     for (size_t i = 0; i < c.meshes.size(); ++i) {
-        c.h_items[i] = BatchItem{c.meshes[i]->plan.view(), X[i], cc[i], vals[i],
-                                 mesh_threshold(c.meshes[i]), 0};
+        BatchItem &it = c.h_items[c.place[i]];
+        it = BatchItem{c.meshes[i]->plan.view(), X[i], cc[i], vals[i], mesh_threshold(c.meshes[i]), 0};
         // the elasticity operator's values: the DOF matrix (bounds of the debug build)
-        if (c.elastic) c.h_items[i].pv.nnz = 9 * c.meshes[i]->nnz - 3 * c.meshes[i]->n_nodes;
+        if (c.elastic) it.pv.nnz = 9 * c.meshes[i]->nnz - 3 * c.meshes[i]->n_nodes;
     }
 }
 
@@ -99,42 +112,76 @@ static fem_status upload_items(BatchCtx &c, cudaStream_t s) {
     return FEM_OK;
 }
 
-static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *const *cc, void *const *vals,
-                             cudaStream_t s) {
+// Cuts the batch into parts (see above): meshes without lists into one, the others into
+// as few as their order gives when each joins the first part that holds it.
+static void make_parts(BatchCtx &c) {
     const int n = (int)c.meshes.size();
+    std::vector<std::vector<int>> of;
+    auto part = [&](bool gather) -> size_t {
+        c.parts.emplace_back();
+        c.parts.back().gather = gather;
+        of.emplace_back();
+        return c.parts.size() - 1;
+    };
+    size_t other = SIZE_MAX;
+    for (int i = 0; i < n; ++i) {
+        const Plan &P = c.meshes[i]->plan;
+        size_t at = SIZE_MAX;
+        if (c.tiles || c.elastic || !P.full.lists.ready) {
+            if (other == SIZE_MAX) other = part(false);
+            at = other;
+        } else {
+            for (size_t q = 0; q < c.parts.size() && at == SIZE_MAX; ++q) {
+                GatherMax gm = c.parts[q].gm;
+                gm.add(P);
+                if (c.parts[q].gather && gather_batch_fits(c.npe, c.mixed, gm)) at = q;
+            }
+            if (at == SIZE_MAX) at = part(true);  // a mesh with lists fits by itself
+            c.parts[at].gm.add(P);
+        }
+        of[at].push_back(i);
+    }
+    c.place.assign(n, 0);
+    c.mesh_at.clear();
+    for (size_t q = 0; q < c.parts.size(); ++q) {
+        c.parts[q].first = (int)c.mesh_at.size();
+        c.parts[q].n = (int)of[q].size();
+        for (int i : of[q]) {
+            c.place[i] = (int)c.mesh_at.size();
+            c.mesh_at.push_back(i);
+        }
+    }
+}
+
+// Tables of one part (its work prefixes, n + 1 each), then its launch: every candidate
+// launch shape is timed on the real batch, the fastest kept.
+static fem_status create_part(BatchCtx &c, int q, cudaStream_t s) {
+    BatchPart &part = c.parts[q];
+    const int n = part.n, base = part.first + q;
     std::vector<int64_t> prefix(n + 1, 0), bprefix(n + 1, 0);
     PlanMax pm;
     TileMax tm;
-    GatherMax gm;
-    for (int i = 0; i < n; ++i) {
+    for (int k = 0; k < n; ++k) {
+        const fem_mesh m = c.meshes[c.mesh_at[part.first + k]];
         if (c.tiles) {
-            prefix[i + 1] = prefix[i] + c.meshes[i]->tiles.n_tiles;
-            bprefix[i + 1] = bprefix[i] + c.meshes[i]->tiles.n_brows;
-            tm.add(c.meshes[i]->tiles);
+            prefix[k + 1] = prefix[k] + m->tiles.n_tiles;
+            bprefix[k + 1] = bprefix[k] + m->tiles.n_brows;
+            tm.add(m->tiles);
         } else {
-            prefix[i + 1] = prefix[i] + c.meshes[i]->plan.n_patches;
-            pm.add(c.meshes[i]->plan);
-            gm.add(c.meshes[i]->plan);
+            prefix[k + 1] = prefix[k] + m->plan.n_patches;
+            pm.add(m->plan);
         }
     }
-    if (c.tiles) FEM_CUDA(cudaMalloc(&c.d_titems, n * sizeof(TileBatchItem)));
-    else FEM_CUDA(cudaMalloc(&c.d_items, n * sizeof(BatchItem)));
-    FEM_CUDA(cudaMalloc(&c.d_prefix, (n + 1) * sizeof(int64_t)));
-    FEM_CUDA(cudaMemcpyAsync(c.d_prefix, prefix.data(), (n + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
-    if (c.tiles) {
-        FEM_CUDA(cudaMalloc(&c.d_bprefix, (n + 1) * sizeof(int64_t)));
-        FEM_CUDA(cudaMemcpyAsync(c.d_bprefix, bprefix.data(), (n + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    FEM_CUDA(cudaMemcpyAsync(c.d_prefix + base, prefix.data(), (n + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, s));
+    if (c.tiles)
+        FEM_CUDA(cudaMemcpyAsync(c.d_bprefix + base, bprefix.data(), (n + 1) * sizeof(int64_t), cudaMemcpyHostToDevice,
+                                 s));
+    if (part.gather) {
+        FEM_CUDA(cudaMalloc(&part.d_gpatch, std::max<int64_t>(prefix[n], 1) * sizeof(GatherPatch)));
+        for (int k = 0; k < n; ++k)
+            FEM_TRY(launch_gather_table(c.meshes[c.mesh_at[part.first + k]]->plan.full.lists.patch.ptr,
+                                        prefix[k + 1] - prefix[k], k, part.d_gpatch + prefix[k], s));
     }
-    if (c.gather) {
-        FEM_CUDA(cudaMalloc(&c.d_gpatch, std::max<int64_t>(prefix[n], 1) * sizeof(GatherPatch)));
-        for (int i = 0; i < n; ++i)
-            FEM_TRY(launch_gather_table(c.meshes[i]->plan.full.lists.patch.ptr, prefix[i + 1] - prefix[i], i,
-                                        c.d_gpatch + prefix[i], s));
-    }
-    c.h_items.resize(n);
-    c.h_titems.resize(n);
-    fill_items(c, X, cc, vals);
-    FEM_TRY(upload_items(c, s));
 
     // tuner: time every candidate launch shape on the real batch, keep the fastest
     const fem_options &o = c.meshes[0]->opt;
@@ -157,23 +204,22 @@ static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *cons
     FEM_CUDA(cudaEventCreate(&e0));
     FEM_CUDA(cudaEventCreate(&e1));
     float best = 1e30f;
-    BatchLaunch best_bl;
     bool have = false;
     for (auto &cd : cands) {
         BatchLaunch bl;
-        bl.items = c.d_items;
-        bl.titems = c.d_titems;
-        bl.bprefix = c.d_bprefix;
-        bl.prefix = c.d_prefix;
-        bl.gpatch = c.d_gpatch;
+        bl.items = c.tiles ? nullptr : c.d_items + part.first;
+        bl.titems = c.tiles ? c.d_titems + part.first : nullptr;
+        bl.bprefix = c.tiles ? c.d_bprefix + base : nullptr;
+        bl.prefix = c.d_prefix + base;
+        bl.gpatch = part.d_gpatch;
         bl.n_work = prefix[n];
         bl.n = n;
         bl.mode = kernel_mode(c.meshes[0]->opt);
         bl.wait = wait_ctl(c.meshes[0]);
         const fem_status cs = c.elastic ? elastic_batched_config(c.npe, c.mixed, pm, cd.first, cd.second, &bl)
                               : c.tiles ? tile_batched_config(c.npe, c.mixed, tm, cd.first, cd.second, &bl)
-                              : c.gather ? gather_batched_config(c.npe, c.mixed, gm, cd.first, cd.second, &bl)
-                                        : batched_config(c.npe, c.mixed, pm, cd.first, cd.second, &bl);
+                              : part.gather ? gather_batched_config(c.npe, c.mixed, part.gm, cd.first, cd.second, &bl)
+                                            : batched_config(c.npe, c.mixed, pm, cd.first, cd.second, &bl);
         if (cs != FEM_OK) continue;
         FEM_TRY(launch_batched_kernel(bl, s));  // warm-up
         float tot = 0.f;
@@ -187,10 +233,9 @@ static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *cons
             FEM_CUDA(cudaEventElapsedTime(&ms, e0, e1));
             tot += ms;
         }
-        ++c.tried;
         if (!have || tot < best) {
             best = tot;
-            best_bl = bl;
+            part.bl = bl;
             have = true;
         }
     }
@@ -200,16 +245,31 @@ static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *cons
         set_error("no launch shape of the batched kernel fits this batch");
         return FEM_ERR_UNSUPPORTED;
     }
-    c.bl = best_bl;
-    c.tuned_ms = best / 3.f;
+    return FEM_OK;
+}
 
-    // capture the launch once
+static fem_status create_ctx(BatchCtx &c, const void *const *X, const void *const *cc, void *const *vals,
+                             cudaStream_t s) {
+    make_parts(c);
+    const size_t n = c.meshes.size(), nq = c.parts.size();
+    if (c.tiles) FEM_CUDA(cudaMalloc(&c.d_titems, n * sizeof(TileBatchItem)));
+    else FEM_CUDA(cudaMalloc(&c.d_items, n * sizeof(BatchItem)));
+    FEM_CUDA(cudaMalloc(&c.d_prefix, (n + nq) * sizeof(int64_t)));
+    if (c.tiles) FEM_CUDA(cudaMalloc(&c.d_bprefix, (n + nq) * sizeof(int64_t)));
+    c.h_items.resize(n);
+    c.h_titems.resize(n);
+    fill_items(c, X, cc, vals);
+    FEM_TRY(upload_items(c, s));
+    for (size_t q = 0; q < nq; ++q) FEM_TRY(create_part(c, (int)q, s));
+
+    // capture the launches once
     cudaStream_t cs;
     FEM_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     fem_status st = FEM_OK;
     if (e == cudaSuccess) {
-        st = launch_batched_kernel(c.bl, cs);
+        for (const BatchPart &part : c.parts)
+            if (st == FEM_OK) st = launch_batched_kernel(part.bl, cs);
         e = cudaStreamEndCapture(cs, &c.graph);
     }
     cudaStreamDestroy(cs);
@@ -247,18 +307,6 @@ fem_status launch_batched(const fem_mesh *ms, int n, bool mixed, bool tiles, con
         set_error("batched builds take %s X and c", mixed ? "float" : "double");
         return FEM_ERR_UNSUPPORTED;
     }
-    // gather lists when every mesh of the batch has them, else the scatter for all
-    // (a mesh planned for it anew leaves the batch cache, so this comes first)
-    bool gather = !tiles && !elastic;
-    for (int i = 0; i < n; ++i) gather = gather && ms[i]->plan.full.lists.ready;
-    if (!gather && !tiles && !elastic)
-        for (int i = 0; i < n; ++i) {
-            FEM_TRY(ensure_targets(ms[i], s));
-            if (ms[i]->plan.chunked) {
-                set_error("mesh %d of the batch is planned in groups under its memory budget", i);
-                return FEM_ERR_UNSUPPORTED;
-            }
-        }
     std::lock_guard<std::mutex> lock(g_batch_mu);
     BatchCtx *ctx = find_ctx(ms, n, mixed, tiles, xd, cd);
     if (!ctx) {
@@ -270,7 +318,6 @@ fem_status launch_batched(const fem_mesh *ms, int n, bool mixed, bool tiles, con
         nc->cd = cd;
         nc->npe = npe;
         nc->elastic = elastic;
-        nc->gather = gather;
         FEM_TRY(create_ctx(*nc, X, c, vals, s));
         if (g_batch_ctx.size() >= MAX_BATCH_CTX) g_batch_ctx.erase(g_batch_ctx.begin());
         g_batch_ctx.push_back(std::move(nc));
@@ -279,7 +326,7 @@ fem_status launch_batched(const fem_mesh *ms, int n, bool mixed, bool tiles, con
     fill_items(*ctx, X, c, vals);
     FEM_TRY(upload_items(*ctx, s));
     FEM_CUDA(cudaGraphLaunch(ctx->exec, s));
-    count_launch();
+    count_launch((int)ctx->parts.size());
     return FEM_OK;
 }
 
@@ -289,9 +336,10 @@ fem_status batched_query(const fem_mesh *ms, int n, bool mixed, int *threads, in
         BatchCtx &c = *p;
         if (c.mixed != mixed || (int)c.meshes.size() != n || !std::equal(c.meshes.begin(), c.meshes.end(), ms))
             continue;
-        if (threads) *threads = c.bl.threads;
-        if (grid) *grid = c.bl.grid;
-        if (blocks_per_sm) *blocks_per_sm = c.bl.grid / num_sms();
+        const BatchLaunch &bl = c.parts[0].bl;  // of a batch in parts: the first mesh's
+        if (threads) *threads = bl.threads;
+        if (grid) *grid = bl.grid;
+        if (blocks_per_sm) *blocks_per_sm = bl.grid / num_sms();
         return FEM_OK;
     }
     set_error("no batched build of these meshes has run");

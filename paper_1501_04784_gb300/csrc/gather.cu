@@ -616,6 +616,15 @@ static fem_status gather_batched_config_t(const GatherMax &gm, int threads, int 
     return FEM_OK;
 }
 
+bool gather_batch_fits(int npe, bool mixed, const GatherMax &gm) {
+    int dev = 0, limit = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return false;
+    const size_t w = mixed ? 4 : 8;
+    return gather_smem_layout(gm, npe, true, w, w, w).total + 1024 <= (size_t)limit;  // (and the static part)
+}
+
 fem_status gather_batched_config(int npe, bool mixed, const GatherMax &gm, int threads, int blocks_per_sm,
                                  BatchLaunch *out) {
     out->npe = npe;

@@ -301,9 +301,6 @@ fem_status ensure_positions(fem_mesh m, cudaStream_t s);
 // Gather lists of a closure (gather_plan.cu), and whether mesh m's builds may run on them.
 fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s);
 bool wants_lists(fem_mesh m);
-// The full closure's accumulator targets (the colour-ordered scatter): plans mesh m
-// again without gather lists when the builds ran on those.
-fem_status ensure_targets(fem_mesh m, cudaStream_t s);
 // One call's use of the mesh's ordered coordinates.  A mixed build writes nothing of the
 // mesh's but its status word, and calls on several streams or threads rely on that, so
 // the buffer passes from call to call: a call's stream waits for the last reader's event,

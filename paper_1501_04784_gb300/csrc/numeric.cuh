@@ -191,6 +191,8 @@ struct BatchLaunch {
 fem_status batched_config(int npe, bool mixed, const PlanMax &pm, int threads, int blocks_per_sm, BatchLaunch *out);
 fem_status launch_batched_kernel(const BatchLaunch &bl, cudaStream_t s);
 
+// Whether meshes with these largest patch sizes fit one launch.
+bool gather_batch_fits(int npe, bool mixed, const GatherMax &gm);
 fem_status gather_batched_config(int npe, bool mixed, const GatherMax &gm, int threads, int blocks_per_sm,
                                  BatchLaunch *out);
 fem_status launch_gather_batched_kernel(const BatchLaunch &bl, cudaStream_t s);

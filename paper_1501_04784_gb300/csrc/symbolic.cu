@@ -1615,17 +1615,6 @@ bool wants_lists(fem_mesh m) {
     return m->opt.operator_kind != 2 && !m->opt.fp64_fused && !m->opt.debug_stall && !m->no_lists;
 }
 
-fem_status ensure_targets(fem_mesh m, cudaStream_t s) {
-    if (!m->plan_built || m->plan.chunked || !m->plan.full.lists.ready) return FEM_OK;
-    m->no_lists = true;
-    batch_forget(m);
-    m->plan_built = false;
-    ArenaKeep keep(m->arena);
-    FEM_TRY(build_plan(m, s));
-    m->plan_built = true;
-    return FEM_OK;
-}
-
 // The closures carry the in-row positions from now on (the backward pass reads
 // them; forward builds do not, so a mesh that only builds K does not hold them).
 // Closures built per patch group get them when they are built; the cached full
