@@ -601,14 +601,16 @@ __device__ __forceinline__ int primary_elems(const PlanView &pv, int npe, int64_
 template <typename T>
 constexpr int vjp_elem_threads() { return sizeof(T) == 8 ? 128 : 256; }
 
-template <int NPE, typename T, typename S, typename CT, bool MASS>
+// X4 (plans with gather lists, FP32 coordinates): a node's coordinates in a 16-byte row of
+// shared memory.  The scatter's closures may need all of it, and keep rows of three.
+template <int NPE, typename T, typename S, typename CT, bool MASS, bool X4>
 __global__ void __launch_bounds__(256) k_vjp_elem(PlanView pv, const int64_t *__restrict__ rowptr,
                                                   const S *__restrict__ X, const float4 *__restrict__ xrank,
                                                   const CT *__restrict__ c, const T *__restrict__ G,
                                                   T *__restrict__ dxe, T *__restrict__ dcout, ElemSmem L,
                                                   int *status) {
     constexpr int NP = NPE * (NPE + 1) / 2;
-    constexpr bool X4 = sizeof(S) == 4;  // FP32 coordinates: one 16-byte row a node
+    static_assert(!X4 || sizeof(S) == 4, "16-byte rows hold FP32 coordinates");
     constexpr int XW = X4 ? 4 : 3;
     extern __shared__ __align__(16) unsigned char vel_smem[];
     __shared__ int n_prim;
@@ -917,11 +919,11 @@ static int grid_for(const void *f, int threads, size_t smem, int64_t np, const c
     return (int)std::max<int64_t>(1, std::min<int64_t>(np, (int64_t)num_sms() * per_sm));
 }
 
-ElemSmem elem_smem(const Plan &P, const Closure &cl, size_t xsize) {
+ElemSmem elem_smem(const Plan &P, const Closure &cl, size_t xrow) {
     ElemSmem L{};
     size_t o = 0;
     L.xs = o;
-    o = a16(o + (size_t)P.max_cnodes * (xsize == 4 ? 16 : 24));
+    o = a16(o + (size_t)P.max_cnodes * xrow);
     L.cown = o;
     o = a16(o + (size_t)P.max_cnodes * 4);
     L.rp = o;
@@ -948,12 +950,12 @@ static fem_status launch_vjp_sum_t(fem_mesh m, const Closure &cl, const void *dx
     return FEM_OK;
 }
 
-template <int NPE, typename T, typename S, typename CT>
-static fem_status launch_vjp_elem_t(fem_mesh m, const Closure &cl, const void *X, const void *c, const void *G,
+template <int NPE, typename T, typename S, typename CT, bool X4>
+static fem_status launch_vjp_elem_x(fem_mesh m, const Closure &cl, const void *X, const void *c, const void *G,
                                     void *dxe, void *dc, cudaStream_t s) {
     const Plan &P = m->plan;
-    const ElemSmem L = elem_smem(P, cl, sizeof(S));
-    auto f = m->opt.operator_kind == 1 ? k_vjp_elem<NPE, T, S, CT, true> : k_vjp_elem<NPE, T, S, CT, false>;
+    const ElemSmem L = elem_smem(P, cl, (X4 ? 4 : 3) * sizeof(S));
+    auto f = m->opt.operator_kind == 1 ? k_vjp_elem<NPE, T, S, CT, true, X4> : k_vjp_elem<NPE, T, S, CT, false, X4>;
     FEM_CUDA(allow_smem(f, L.total));
     if constexpr (NPE == 4) {
         // tets: shared memory for two blocks per SM, the rest of the unified L1/shared
@@ -974,14 +976,21 @@ static fem_status launch_vjp_elem_t(fem_mesh m, const Closure &cl, const void *X
         if (cl.lists.ready && (P.id_runs || m->nnz * (int64_t)sizeof(T) <= (128 << 20))) nt = 128;
     const int grid = grid_for((const void *)f, nt, L.total, np, "backward element kernel", &st);
     if (st != FEM_OK) return st;
-    const XrankUse ordered(m, sizeof(T) == 4, sizeof(S) == 4 ? FEM_F32 : FEM_F64, s);
+    const XrankUse ordered(m, X4, FEM_F32, s);
     const float4 *xr = reinterpret_cast<const float4 *>(ordered.ptr());
-    if constexpr (sizeof(S) == 4)
-        if (xr) FEM_TRY(launch_order_x(P, (const float *)X, ordered.ptr(), s));
+    if (xr) FEM_TRY(launch_order_x(P, (const float *)X, ordered.ptr(), s));
     f<<<grid, nt, L.total, s>>>(P.view(cl), m->rowptr.ptr, (const S *)X, xr, (const CT *)c, (const T *)G, (T *)dxe,
                                 (T *)dc, L, m->status.ptr);
     FEM_LAUNCHED("k_vjp_elem");
     return FEM_OK;
+}
+
+template <int NPE, typename T, typename S, typename CT>
+static fem_status launch_vjp_elem_t(fem_mesh m, const Closure &cl, const void *X, const void *c, const void *G,
+                                    void *dxe, void *dc, cudaStream_t s) {
+    if constexpr (sizeof(S) == 4)
+        if (cl.lists.ready) return launch_vjp_elem_x<NPE, T, S, CT, true>(m, cl, X, c, G, dxe, dc, s);
+    return launch_vjp_elem_x<NPE, T, S, CT, false>(m, cl, X, c, G, dxe, dc, s);
 }
 
 template <int NPE, typename T>
@@ -1070,10 +1079,22 @@ static fem_status launch_vjp_group(fem_mesh m, const Closure &cl, bool mixed, co
 #undef FEM_V
 }
 
+// Whether the largest closure fits k_vjp_elem's shared memory.  Thin meshes' patches
+// touch many nodes an element (300 x 300 x 4 cells in tetrahedra: 5,930 nodes in a
+// closure, 235 KB with FP64 coordinates); the fused kernel keeps 4 bytes a node less.
+static bool vjp_elem_fits(fem_mesh m, fem_dtype xd) {
+    int dev = 0, limit = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return false;
+    const size_t row = xd == FEM_F64 ? 24 : m->plan.full.lists.ready ? 16 : 12;
+    return elem_smem(m->plan, m->plan.full, row).total + 64 <= (size_t)limit;  // (and the static part)
+}
+
 fem_status launch_vjp(fem_mesh m, bool mixed, const void *X, fem_dtype xd, const void *c, fem_dtype cd,
                       const void *G, void *dX, void *dc, cudaStream_t s) {
     void *dxe = nullptr;
-    const fem_status st = vjp_scratch(m, !mixed, &dxe);
+    const fem_status st = vjp_elem_fits(m, xd) ? vjp_scratch(m, !mixed, &dxe) : FEM_ERR_BUDGET;
     if (st == FEM_OK) {
         FEM_TRY(for_each_group(m, s, [&](const Closure &cl) {
             return launch_vjp_elem(m, cl, mixed, X, xd, c, cd, G, dxe, dc, s);
