@@ -791,6 +791,17 @@ fem_status fem_batched_config(const fem_mesh *meshes, int n, fem_prec p, int *bl
     return batched_query(meshes, n, p == FEM_MIXED, block_threads, blocks_per_sm, grid);
 }
 
+// Under a budget, library memory that calls take as they need it must not decide how the
+// next plan is made: the FP64 matrices and the host builds' staging are given back (and
+// taken again by the calls that use them).
+static void make_room(fem_mesh m) {
+    if (!m->arena.budget) return;
+    cudaDeviceSynchronize();
+    m->ke64.free();
+    m->chunk_slots.free();
+    for (auto &slot : m->host_stage) slot.free();
+}
+
 // Tuner of the assembly tile and of the threads per block: the plan is rebuilt
 // for each candidate size (elements per tile when the builds run on tiles,
 // lower-CSR entries per patch otherwise) and every candidate is timed on the
@@ -819,7 +830,11 @@ fem_status fem_autotune(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype
     const int *sizes = tiles ? (m->npe == 8 ? tiles_brick : tiles_tet)
                              : (is_elastic(m) ? entries_elastic : entries_scalar);
     const int *threads = is_elastic(m) ? threads_elastic : threads_scalar;
+    DevBuf<unsigned char> flush;
+    const size_t flush_bytes = (size_t)256 << 20;
     auto replan = [&](cudaStream_t st) -> fem_status {
+        make_room(m);
+        if (m->arena.budget) flush.free();
         if (tiles) return build_tiles(m, st);
         fem_status r = build_plan(m, st);
         if (r == FEM_OK) m->plan_built = true;
@@ -833,9 +848,6 @@ fem_status fem_autotune(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype
     // Candidates are timed from a cold L2, as a build that follows other work
     // sees it: a 256 MB scratch (twice the L2) is rewritten before every timed
     // build, when the memory budget has room for it.  Median of 5 builds.
-    DevBuf<unsigned char> flush;
-    const size_t flush_bytes = (size_t)256 << 20;
-    if (flush.alloc(m->arena, flush_bytes, "tuner L2 flush") != FEM_OK) cudaGetLastError();
     for (int ie = 0; ie < 5; ++ie) {
         const int pe = sizes[ie];
         if (ie > 0 && pe == sizes[ie - 1]) continue;
@@ -854,6 +866,7 @@ fem_status fem_autotune(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype
                 break;
             }
             if (fem_build_K(m, p, X, x_dtype, c, c_dtype, vals, stream) != FEM_OK) continue;
+            if (!flush.ptr && flush.alloc(m->arena, flush_bytes, "tuner L2 flush") != FEM_OK) cudaGetLastError();
             float rep[5];
             for (int r = 0; r < 5; ++r) {
                 if (flush.ptr) FEM_CUDA(cudaMemsetAsync(flush.ptr, r, flush_bytes, s));
@@ -910,6 +923,7 @@ fem_status fem_set_tuning(fem_mesh m, int patch_entries, int block_threads, void
     cudaStream_t s = as_stream(stream);
     ArenaKeep keep(m->arena);
     fem_status st = FEM_OK;
+    make_room(m);
     if (use_tiles(m)) {
         st = build_tiles(m, s);
     } else if (m->plan_built) {

@@ -233,7 +233,8 @@ struct fem_mesh_s {
     fem::DevBuf<int32_t> inc_elem;
     fem::Plan plan;
     bool plan_built = false;  // the patch plan exists (it is built on first use when tiles serve the builds)
-    bool no_lists = false;    // the builds run on the colour-ordered scatter, not on gather lists
+    bool lone_node = false;   // a node has no element: gather lists hold a diagonal for every row
+    bool lists_off = false;   // the present plan was made without gather lists (decided anew by each plan)
     bool want_pos = false;    // closures carry the in-row positions (set by the first backward pass)
     fem::TilePlan tiles;      // element tiles of the scalar operators (tile.cuh)
     // device status word: set by a bounded device-side wait that gave up

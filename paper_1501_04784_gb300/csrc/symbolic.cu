@@ -1074,7 +1074,7 @@ fem_status build_pattern(fem_mesh m, cudaStream_t s) {
         FEM_CUDA(cudaMemcpyAsync(h, mx.ptr, sizeof(h), cudaMemcpyDeviceToHost, s));
         FEM_CUDA(cudaStreamSynchronize(s));
         max_deg = h[0];
-        if (h[1]) m->no_lists = true;  // gather lists hold a diagonal for every row
+        m->lone_node = h[1] != 0;
     }
     m->max_deg = (int64_t)max_deg;
     const int cap = (int)(max_deg * npe);
@@ -1596,7 +1596,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         if (cl.lists.ready) {
             // coordinates in locality order, filled by each mixed call (refused by the
             // budget: the kernels gather them from X)
-            if (m->n_nodes >= XRANK_MIN && !P.id_runs && m->xrank.n < 4 * (size_t)m->n_nodes &&
+            if (m->n_nodes >= XRANK_MIN && !P.id_runs &&
                 m->xrank.alloc(ar, 4 * (size_t)m->n_nodes, "ordered X") != FEM_OK)
                 cudaGetLastError();
             return FEM_OK;
@@ -1612,7 +1612,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
 // Gather lists serve the scalar operators' builds; the fused FP64 form and the
 // kernels' test modes run on the colour-ordered scatter.
 bool wants_lists(fem_mesh m) {
-    return m->opt.operator_kind != 2 && !m->opt.fp64_fused && !m->opt.debug_stall && !m->no_lists;
+    return m->opt.operator_kind != 2 && !m->opt.fp64_fused && !m->opt.debug_stall && !m->lone_node && !m->lists_off;
 }
 
 // The closures carry the in-row positions from now on (the backward pass reads
@@ -1876,6 +1876,10 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
     int dev = 0, limit = 0;
     FEM_CUDA(cudaGetDevice(&dev));
     FEM_CUDA(cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    // another stream may still run on the plan that goes: its ranges are used again here
+    if (m->plan.n_patches > 0) FEM_CUDA(cudaDeviceSynchronize());
+    m->xrank.free();  // the new plan has its own, if any
+    m->lists_off = false;
     int64_t cap = 0;
     for (;;) {
         const fem_status st = build_plan_cap(m, s, cap);
@@ -1886,7 +1890,7 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
         if (cap == 0 && (st == FEM_OK || st == FEM_ERR_BUDGET) && wants_lists(m) && !m->plan.full.lists.ready &&
             default_list_patches(m)) {
             cudaGetLastError();
-            m->no_lists = true;
+            m->lists_off = true;
             continue;
         }
         FEM_TRY(st);
