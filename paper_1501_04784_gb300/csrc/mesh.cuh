@@ -302,6 +302,10 @@ fem_status ensure_positions(fem_mesh m, cudaStream_t s);
 // Gather lists of a closure (gather_plan.cu), and whether mesh m's builds may run on them.
 fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s);
 bool wants_lists(fem_mesh m);
+// Whether the budget holds the pattern and `plan` bytes beside what the calls may take later.
+bool budget_holds(fem_mesh m, size_t plan);
+// Nodes from which single meshes' FP32 coordinates are put in locality order (symbolic.cu).
+bool wants_ordered_x(fem_mesh m);
 // One call's use of the mesh's ordered coordinates.  A mixed build writes nothing of the
 // mesh's but its status word, and calls on several streams or threads rely on that, so
 // the buffer passes from call to call: a call's stream waits for the last reader's event,

@@ -1596,7 +1596,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         if (cl.lists.ready) {
             // coordinates in locality order, filled by each mixed call (refused by the
             // budget: the kernels gather them from X)
-            if (m->n_nodes >= XRANK_MIN && !P.id_runs &&
+            if (wants_ordered_x(m) &&
                 m->xrank.alloc(ar, 4 * (size_t)m->n_nodes, "ordered X") != FEM_OK)
                 cudaGetLastError();
             return FEM_OK;
@@ -1607,6 +1607,26 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
     }
     FEM_TRY(cl.celem_aidx.alloc(ar, nce * (m->np / 2), "celem accumulator targets"));
     return fill();
+}
+
+bool wants_ordered_x(fem_mesh m) { return m->n_nodes >= XRANK_MIN && !m->plan.id_runs; }
+
+// Lists are about a fifth of a plan (27M bricks: 9.83 GB with them, 8.10 without) and only
+// make builds faster; the library memory that calls take as they need it decides whether
+// they can run, or whether FP64 builds and backward passes run staged.  So under a budget
+// lists are taken only where all of that fits beside them: the FP64 element matrices (or
+// the backward's element gradients, in the same buffer), the host builds' three staging
+// slots, the tiles' partial rows, the tuner's scratch.  It depends on the mesh and the
+// budget alone, not on what is held when a plan is made.
+bool budget_holds(fem_mesh m, size_t plan) {
+    if (!m->arena.budget) return true;
+    const size_t N = (size_t)m->n_nodes, nel = (size_t)m->n_elems, nnz = (size_t)m->nnz;
+    const size_t pattern = m->rowptr.bytes() + m->col.bytes() + m->inc_ptr.bytes() + m->inc_elem.bytes() +
+                           m->order.bytes() + m->tiles.bytes();
+    const size_t staged = nel * (size_t)std::max(m->np, 3 * m->npe) * sizeof(double);
+    const size_t host = fem_mesh_s::HOST_STAGES * (24 * N + 8 * nel + 8 * nnz + 1024);
+    const size_t partial = m->tiles.ready ? (size_t)m->tiles.partial_n * sizeof(double) : 0;
+    return pattern + plan + staged + host + partial + ((size_t)256 << 20) <= m->arena.budget;
 }
 
 // Gather lists serve the scalar operators' builds; the fused FP64 form and the
@@ -1879,7 +1899,7 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
     // another stream may still run on the plan that goes: its ranges are used again here
     if (m->plan.n_patches > 0) FEM_CUDA(cudaDeviceSynchronize());
     m->xrank.free();  // the new plan has its own, if any
-    m->lists_off = false;
+    m->lists_off = !budget_holds(m, 0);
     int64_t cap = 0;
     for (;;) {
         const fem_status st = build_plan_cap(m, s, cap);

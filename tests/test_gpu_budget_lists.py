@@ -47,3 +47,61 @@ def test_tuning_keeps_the_lists(fem, case, room, prec):
     assert (after["n_patches"], after["n_groups"]) == (before["n_patches"], before["n_groups"])
     assert torch.equal(mesh.build_K(X.to(dt), c.to(dt), prec), want)
     mesh.sync()
+
+
+@pytest.mark.parametrize("room", [0, MB, 12 * MB])
+def test_lists_leave_room_for_staging(fem, case, room):
+    """A budget that holds the scatter's plan and the call's staging is enough."""
+    m, E, X, c = case
+    Xh, ch = X.cpu(), c.cpu()  # pageable: K's values need device staging
+    # planned for the scatter, its memory counted as under a budget (not in slabs)
+    plain = fem.Mesh(E, m.n_nodes, X=X, fp64_fused=1, mem_budget_bytes=1 << 40)
+    plain.pattern()
+    want = plain.build_K_host(Xh, ch, "mixed", out=torch.empty(plain.nnz))
+    X64, c64 = X.double(), c.double()
+    G = torch.randn(plain.nnz, device="cuda", dtype=torch.float64)
+    plain.vjp(X64, c64, G, "fp64")  # the in-row positions and the staged gradients (24 values a brick)
+    budget = plain.info()["live_bytes"] + m.n_elems * (36 - 24) * 8 + room
+    mesh = fem.Mesh(E, m.n_nodes, X=X, mem_budget_bytes=budget)
+    mesh.pattern()
+    assert mesh.info()["n_groups"] == 1
+    v = mesh.build_K_host(Xh, ch, "mixed", out=torch.empty(mesh.nnz))
+    assert float((v - want).abs().max()) <= 4e-6 * float(want.abs().max())
+    # FP64 builds and backward passes run staged (two launches each), as without a budget
+    mesh.build_K(X64, c64, "fp64")
+    mesh.vjp(X64, c64, G, "fp64")
+    for call in (lambda: mesh.build_K(X64, c64, "fp64"), lambda: mesh.vjp(X64, c64, G, "fp64")):
+        fem.launch_count(reset=True)
+        call()
+        assert fem.launch_count() == 2
+    assert mesh.info()["peak_bytes"] <= budget
+    mesh.sync()
+
+
+def test_ordered_coordinates_under_a_budget(fem):
+    """A permuted mesh of 2^18 nodes: builds, then the first backward pass, within budgets
+    that hold the scatter's plan and staging, and with lists where all of it fits."""
+    m = meshgen.hex_grid(66, 64, 62, jitter=0.2, permute_nodes=True)
+    E, X, c = dev(m.E, torch.int32), dev(m.X, torch.float32), dev(m.c, torch.float32)
+    free = fem.Mesh(E, m.n_nodes, X=X)
+    plain = fem.Mesh(E, m.n_nodes, X=X, fp64_fused=1, mem_budget_bytes=1 << 40)
+    want, _ = free.build_K(X, c, "mixed"), plain.build_K(X, c, "mixed")
+    G = torch.randn(free.nnz, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    dX, dc = free.vjp(X, c, G, "mixed")
+    plain.vjp(X, c, G, "mixed")
+    lists, scatter = free.info()["n_patches"], plain.info()["n_patches"]
+    assert lists > scatter
+    seen = set()
+    for extra in (0, 4, 16, 64, 1024):
+        budget = plain.info()["peak_bytes"] + extra * MB
+        mesh = fem.Mesh(E, m.n_nodes, X=X, mem_budget_bytes=budget)
+        v = mesh.build_K(X, c, "mixed")
+        planned = mesh.info()["n_patches"]
+        assert float((v - want).abs().max()) <= 4e-6 * float(want.abs().max())
+        for u, w in zip(mesh.vjp(X, c, G, "mixed"), (dX, dc)):
+            assert float((u - w).abs().max()) <= 4e-6 * float(w.abs().max())
+        info = mesh.info()
+        assert info["n_groups"] == 1 and info["n_patches"] == planned and info["peak_bytes"] <= budget
+        seen.add(planned)
+        mesh.sync()
+    assert seen == {lists, scatter}
