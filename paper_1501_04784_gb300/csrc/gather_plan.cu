@@ -307,18 +307,20 @@ __global__ void __launch_bounds__(512) k_gather_lists(PlanView pv, const int32_t
     }
 }
 
-// Whether closure cl's patches fit the gather kernels: the largest layout is the
-// fused FP64 one (the batched FP64 builds), and positions are 16-bit.
-static bool gather_fits(const Plan &P, const Closure &cl, int npe, const GatherPlanSmem &L) {
-    const int np = npe * (npe + 1) / 2;
+// The largest layout is the fused FP64 one (the batched FP64 builds), and positions are
+// 16-bit.  A closure holds at least the nodes its patch owns.
+bool lists_fit(fem_mesh m, const Closure &cl) {
+    const Plan &P = m->plan;
     int dev = 0, limit = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&limit, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return false;
     GatherMax gm;
-    gm.add(P);
-    return cl.max_celems * np < 65536 && P.max_own < 32767 &&
-           gather_smem_layout(gm, npe, true, 8, 8, 8).total + 1024 <= (size_t)limit && L.total + 1024 <= (size_t)limit;
+    gm.max_acc = P.max_acc, gm.max_own = P.max_own;
+    gm.max_cnodes = std::max(cl.max_cnodes, P.max_own), gm.max_celems = cl.max_celems;
+    return cl.max_celems * m->np < 65536 && P.max_own < 32767 &&
+           gather_smem_layout(gm, m->npe, true, 8, 8, 8).total + 1024 <= (size_t)limit &&
+           gather_plan_smem(P, cl, m->npe).total + 1024 <= (size_t)limit;
 }
 
 // Builds the lists of the full closure (all patches); leaves lists.ready false when
@@ -330,7 +332,7 @@ fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s) {
     G.free();
     const GatherPlanSmem L = gather_plan_smem(P, cl, m->npe);
     P.max_cnodes = cl.max_cnodes, P.max_celems = cl.max_celems;
-    if (cl.total_celems == 0 || !gather_fits(P, cl, m->npe, L)) return FEM_OK;
+    if (cl.total_celems == 0 || !lists_fit(m, cl)) return FEM_OK;
     const int64_t np_ = cl.p1 - cl.p0;
     const int np = m->npe * (m->npe + 1) / 2;
     G.zero = (int)(cl.max_celems * np);

@@ -299,6 +299,12 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
                          bool with_lists);
 // From now on the closures carry the in-row positions the backward pass reads.
 fem_status ensure_positions(fem_mesh m, cudaStream_t s);
+// Whether a closure's patches fit the gather kernels, by what is known of it (its largest
+// patch, then its longest node list).
+bool lists_fit(fem_mesh m, const Closure &cl);
+// Answer of build_closure to a plan whose patches have the lists' default size and do not
+// fit them: to be made again for the scatter.
+constexpr fem_status PLAN_AGAIN = static_cast<fem_status>(1000);
 // Gather lists of a closure (gather_plan.cu), and whether mesh m's builds may run on them.
 fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s);
 bool wants_lists(fem_mesh m);

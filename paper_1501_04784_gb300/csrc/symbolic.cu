@@ -1306,6 +1306,11 @@ __global__ void __launch_bounds__(512) k_patch_color_order(const uint64_t *ckeys
     }
 }
 
+// Whether patches for gather lists take the size that suits them (build_plan_cap).
+static bool default_list_patches(fem_mesh m) {
+    return m->opt.patch_entries <= 0 || (m->opt.patch_entries > 3072 && m->opt.patch_entries <= 4096);
+}
+
 fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaStream_t s, bool with_pos,
                          bool with_lists) {
     Arena &ar = m->arena;
@@ -1404,6 +1409,14 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
     }
     cl.total_celems = nce;
     for (int64_t p = 0; p < np_; ++p) cl.max_celems = std::max(cl.max_celems, h_pe[p + 1] - h_pe[p]);
+    // One patch out of the lists' range is enough to plan again for the scatter, so that is
+    // found out here, before the closures are coloured and filled: planning a 300 x 300 x 11
+    // mesh to the end first cost 4.5 ms of its 12.7 (thin and stretched meshes: a closure
+    // of the lists' patches holds up to three times what a cube's does).
+    if (with_lists && !lists_fit(m, cl)) {
+        if (default_list_patches(m)) return PLAN_AGAIN;
+        with_lists = false;
+    }
 
     // ---- colouring of each closure (in sweep order), then order each closure by (colour, element)
     if (!swept) {
@@ -1431,7 +1444,7 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         std::swap(ckeys.n, swk.n);
         std::swap(ckeys.arena, swk.arena);
     }
-    {
+    auto colour = [&]() -> fem_status {
         DevBuf<uint8_t> color;
         DevBuf<int> mxc;
         FEM_TRY(color.alloc(ar, nce, "colours"));
@@ -1488,7 +1501,11 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         std::swap(ckeys.ptr, ck2.ptr);
         std::swap(ckeys.n, ck2.n);
         std::swap(ckeys.arena, ck2.arena);
-    }
+        return FEM_OK;
+    };
+    // a plan for lists first learns its closures' node counts, which may end it
+    const bool nodes_first = with_lists;
+    if (!nodes_first) FEM_TRY(colour());
 
     // ---- closure nodes of each patch: ascending ids, or for the gather kernels
     // ascending ranks in the locality order, so that a patch's own nodes are one run
@@ -1528,6 +1545,8 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
         FEM_CUDA(cudaMemcpyAsync(&h_ovf, ovf.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
         FEM_CUDA(cudaStreamSynchronize(s));
         if (!h_ovf) {
+            for (int64_t n : h_cnt) cl.max_cnodes = std::max(cl.max_cnodes, n);
+            if (with_lists && default_list_patches(m) && !lists_fit(m, cl)) return PLAN_AGAIN;
             for (int64_t p = 0; p < np_; ++p) h_off[p + 1] = h_off[p] + h_cnt[p];
             ncn = h_off[np_];
             FEM_TRY(pc.alloc(ar, np_ + 1, "closure node offsets"));
@@ -1560,6 +1579,8 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
                                               rank.ptr ? P.own_row.ptr : nullptr, cl.cnode_gid.ptr, cl.cnode_own.ptr,
                                               cl.cnode_rank.ptr);
     FEM_LAUNCHED("k_cnode_own");
+
+    if (nodes_first) FEM_TRY(colour());
 
     // ---- per closure element data
     FEM_TRY(cl.celem_id.alloc(ar, nce, "celem id"));
@@ -1706,11 +1727,6 @@ static fem_status plan_groups(fem_mesh m, cudaStream_t s) {
         P.n_colors = std::max(P.n_colors, cl.n_colors);
         return FEM_OK;
     });
-}
-
-// Whether patches for gather lists take the size that suits them (build_plan_cap).
-static bool default_list_patches(fem_mesh m) {
-    return m->opt.patch_entries <= 0 || (m->opt.patch_entries > 3072 && m->opt.patch_entries <= 4096);
 }
 
 // Global part of the plan (patches of consecutive nodes in locality order, the
@@ -1904,12 +1920,16 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
     for (;;) {
         const fem_status st = build_plan_cap(m, s, cap);
         // Patches of a size chosen for the gather lists, but no lists (the budget refuses
-        // them, or a closure is out of their range): planned again at the scatter's size
+        // them): planned again at the scatter's size
         // (27M bricks in the patch groups of a 7 GB budget: 57 ms a build at the lists'
         // size, 51 at the scatter's).
         if (cap == 0 && (st == FEM_OK || st == FEM_ERR_BUDGET) && wants_lists(m) && !m->plan.full.lists.ready &&
             default_list_patches(m)) {
             cudaGetLastError();
+            m->lists_off = true;
+            continue;
+        }
+        if (st == PLAN_AGAIN) {
             m->lists_off = true;
             continue;
         }
