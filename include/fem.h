@@ -212,7 +212,9 @@ typedef struct {
     size_t peak_bytes;           /* the most it has held at once */
     int32_t n_chunks;            /* row ranges of the host pipeline (fem_options.host_chunks;
                                     1 = none) */
-    int32_t reserved0;
+    int32_t gather_lists;        /* 1 = the builds sum each entry along lists made with the plan
+                                    (scalar operators, where the lists fit a block's shared
+                                    memory and the budget); 0 = the colour-ordered scatter */
     int64_t tile_rows;           /* rows summed in tiles (a row in k tiles counts k times) */
     int64_t border_rows;         /* rows whose elements span several tiles */
     int64_t partial_values;      /* values of the border rows' partial sums */

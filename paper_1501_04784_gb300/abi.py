@@ -39,7 +39,7 @@ class fem_info(ctypes.Structure):
                 ("max_row_len", ctypes.c_int32), ("plan_bytes", ctypes.c_size_t),
                 ("budget_bytes", ctypes.c_size_t), ("n_groups", ctypes.c_int32),
                 ("assembly", ctypes.c_int32), ("live_bytes", ctypes.c_size_t), ("peak_bytes", ctypes.c_size_t),
-                ("n_chunks", ctypes.c_int32), ("reserved0", ctypes.c_int32), ("tile_rows", ctypes.c_int64),
+                ("n_chunks", ctypes.c_int32), ("gather_lists", ctypes.c_int32), ("tile_rows", ctypes.c_int64),
                 ("border_rows", ctypes.c_int64),
                 ("partial_values", ctypes.c_int64)]
 

@@ -973,6 +973,7 @@ fem_status fem_mesh_info(fem_mesh m, fem_info *info) {
         info->max_patch_cnodes = m->plan.max_cnodes;
         info->max_patch_elems = m->plan.max_celems;
         info->n_colors = m->plan.n_colors;
+        info->gather_lists = m->plan.full.lists.ready ? 1 : 0;
     }
     info->max_row_len = m->max_row_len;
     info->plan_bytes = m->plan.bytes() + m->tiles.bytes() + m->rowptr.bytes() + m->col.bytes() + m->inc_ptr.bytes() +

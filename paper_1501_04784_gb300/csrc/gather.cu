@@ -280,6 +280,10 @@ __device__ __forceinline__ void gather_patches(const PlanView &pv0, const S *__r
         g_wait();
         for (int j = tid; j < d.n_cnodes; j += nthr) {
             int64_t g = gid[j];
+#ifdef FEM_DEBUG_BOUNDS
+            // testing the checks: one planted out-of-range node id per patch
+            if ((mode & PLANT_ID) && j == 0) g = pv.n_nodes;
+#endif
             if (!FEM_IN_BOUNDS(g >= 0 && g < pv.n_nodes, status)) g = 0;
             if (Xr) {
                 g_cp16(&xs[j][0], Xr + g);

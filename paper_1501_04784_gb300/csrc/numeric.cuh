@@ -38,6 +38,8 @@ struct PatchSmem {
 // fem_options.fp64_sums, fp64_dets) and OP_MASS (fem_options.operator_kind: the
 // mass matrix instead of the stiffness matrix).
 static constexpr unsigned FP64_SUMS = 1u, FP64_DETS = 2u, OP_MASS = 4u;
+// Bounds-check build: the gather kernels plant an out-of-range node id (debug_stall 2).
+static constexpr unsigned PLANT_ID = 8u;
 
 // Device-side waits of the patch kernels (colour phases on mbarriers): each wait
 // polls at most `spins` times, then records the failure in *status (read by
@@ -205,7 +207,8 @@ WaitCtl wait_ctl(fem_mesh m);
 fem_status check_status(fem_mesh m, cudaStream_t s);
 
 inline unsigned kernel_mode(const fem_options &o) {
-    return (o.fp64_sums ? FP64_SUMS : 0u) | (o.fp64_dets ? FP64_DETS : 0u) | (o.operator_kind == 1 ? OP_MASS : 0u);
+    return (o.fp64_sums ? FP64_SUMS : 0u) | (o.fp64_dets ? FP64_DETS : 0u) | (o.operator_kind == 1 ? OP_MASS : 0u) |
+           (o.debug_stall == 2 ? PLANT_ID : 0u);
 }
 fem_status launch_patch(const PatchArgs &a, cudaStream_t s);
 

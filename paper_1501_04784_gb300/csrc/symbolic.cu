@@ -1651,9 +1651,9 @@ bool budget_holds(fem_mesh m, size_t plan) {
 }
 
 // Gather lists serve the scalar operators' builds; the fused FP64 form and the
-// kernels' test modes run on the colour-ordered scatter.
+// test of the phase waits run on the colour-ordered scatter.
 bool wants_lists(fem_mesh m) {
-    return m->opt.operator_kind != 2 && !m->opt.fp64_fused && !m->opt.debug_stall && !m->lone_node && !m->lists_off;
+    return m->opt.operator_kind != 2 && !m->opt.fp64_fused && m->opt.debug_stall != 1 && !m->lone_node && !m->lists_off;
 }
 
 // The closures carry the in-row positions from now on (the backward pass reads

@@ -35,6 +35,7 @@ def test_mixed_batch_leaves_the_plans_alone(fem, kind, prec):
     for m in mesh:
         m.pattern()
     before = [m.info() for m in mesh]
+    assert [i["gather_lists"] for i in before] == [1, 0, 1]
     want = [m.build_K(x, k, prec).clone() for m, x, k in zip(mesh, X, c)]
     order = [0, 1, 2, 1, 0]
     for _ in range(2):
@@ -66,7 +67,7 @@ def test_meshes_that_fit_alone_only(fem):
     # element matrices of the cube's closures and the chain's coordinates and ids alone
     # are more than the 227 KB a block can have
     need = 288 * max(i["max_patch_elems"] for i in info) + 28 * max(i["max_patch_cnodes"] for i in info)
-    assert need > 205 << 10
+    assert need > 205 << 10 and all(i["gather_lists"] for i in info)
     for m, x, k, v in zip(mesh, X, c, fem.build_K_batched(mesh, X, c, "fp64")):
         ref = m.build_K(x, k, "fp64")
         assert float((v - ref).abs().max()) <= 1.6e-13 * float(ref.abs().max())

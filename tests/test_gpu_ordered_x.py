@@ -51,6 +51,8 @@ def test_forward_and_backward(fem, case):
     a = fem.Mesh(E, m.n_nodes, X=X, patch_entries=2816 if m.E.shape[1] == 8 else 1024)
     b = fem.Mesh(E, m.n_nodes, X=X, patch_entries=2816 if m.E.shape[1] == 8 else 1024, fp64_fused=1)
     a.pattern()
+    b.pattern()
+    assert a.info()["gather_lists"] == 1 and b.info()["gather_lists"] == 0
     G = torch.randn(a.nnz, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
     for x, c in zip(Xs, cs):
         n, v = launches(fem, lambda: a.build_K(x, c, "mixed"))
