@@ -206,10 +206,10 @@ typedef struct {
                                     tiles, closure_elems = n_elems, max_patch_entries = the
                                     largest tile's accumulator entries, max_patch_cnodes its
                                     rows) */
-    size_t live_bytes;           /* device bytes the library holds for the mesh now (without
-                                    a budget: whole slabs of up to 64 MB that its buffers
-                                    are carved from) */
-    size_t peak_bytes;           /* the most it has held at once */
+    size_t live_bytes;           /* device bytes in the mesh's buffers now (without a budget they
+                                    are carved from slabs of up to 64 MB; what a slab has left
+                                    is not counted) */
+    size_t peak_bytes;           /* the most they have been */
     int32_t n_chunks;            /* row ranges of the host pipeline (fem_options.host_chunks;
                                     1 = none) */
     int32_t gather_lists;        /* 1 = the builds sum each entry along lists made with the plan

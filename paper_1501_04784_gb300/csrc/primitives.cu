@@ -72,7 +72,7 @@ fem_status Arena::alloc(void **p, size_t bytes, const char *what) {
         return FEM_ERR_BUDGET;
     }
     cudaError_t e = cudaMalloc(p, need);
-    if (e != cudaSuccess && !pool.empty()) {
+    if (e != cudaSuccess && !(pool.empty() && slabs.empty())) {  // (an empty slab's bytes count too)
         cudaGetLastError();
         trim();
         e = cudaMalloc(p, need);
