@@ -452,9 +452,7 @@ def run_ours(args):
     alg = algorithmic_bytes(m.n_nodes, m.n_elems, 8, nnz, 4, 4, 4)
     alg64 = algorithmic_bytes(m.n_nodes, m.n_elems, 8, nnz, 8, 8, 8)
     achieved = alg / (ms_step / 1e3) / 1e9
-    # patches of up to 4,096 entries run on gather lists, larger ones on the colour-ordered scatter
-    lists = tuning.get("patch_entries", 0) <= 4096
-    kernel = "k_tile" if info["assembly"] == 1 else "k_gather" if lists else "k_patch"
+    kernel = "k_tile" if info["assembly"] == 1 else "k_gather" if info["gather_lists"] else "k_patch"
     wkey = f"hex8_n{args.n}_mixed_{'t' if info['assembly'] == 1 else 'p'}{tuning.get('patch_entries', 0)}"
     sm_mhz = (clocks or {}).get("sm_mhz") or 2070.0
     alu_peak = SMS * FP32_LANES * 2 * sm_mhz * 1e6 / 1e12          # TFLOP/s at the sampled clock

@@ -921,9 +921,9 @@ fem_status fem_set_tuning(fem_mesh m, int patch_entries, int block_threads, void
     m->opt.blocks_per_sm = 0;
     if (!m->has_pattern) return FEM_OK;  // fem_pattern will plan with these settings
     cudaStream_t s = as_stream(stream);
+    make_room(m);
     ArenaKeep keep(m->arena);
     fem_status st = FEM_OK;
-    make_room(m);
     if (use_tiles(m)) {
         st = build_tiles(m, s);
     } else if (m->plan_built) {

@@ -1639,15 +1639,29 @@ bool wants_ordered_x(fem_mesh m) { return m->n_nodes >= XRANK_MIN && !m->plan.id
 // the backward's element gradients, in the same buffer), the host builds' three staging
 // slots, the tiles' partial rows, the tuner's scratch.  It depends on the mesh and the
 // budget alone, not on what is held when a plan is made.
-bool budget_holds(fem_mesh m, size_t plan) {
-    if (!m->arena.budget) return true;
+static size_t later_needs(fem_mesh m) {
     const size_t N = (size_t)m->n_nodes, nel = (size_t)m->n_elems, nnz = (size_t)m->nnz;
-    const size_t pattern = m->rowptr.bytes() + m->col.bytes() + m->inc_ptr.bytes() + m->inc_elem.bytes() +
-                           m->order.bytes() + m->tiles.bytes();
     const size_t staged = nel * (size_t)std::max(m->np, 3 * m->npe) * sizeof(double);
     const size_t host = fem_mesh_s::HOST_STAGES * (24 * N + 8 * nel + 8 * nnz + 1024);
     const size_t partial = m->tiles.ready ? (size_t)m->tiles.partial_n * sizeof(double) : 0;
-    return pattern + plan + staged + host + partial + ((size_t)256 << 20) <= m->arena.budget;
+    return staged + host + partial + ((size_t)256 << 20);
+}
+
+bool budget_holds(fem_mesh m, size_t plan) {
+    const size_t pattern = m->rowptr.bytes() + m->col.bytes() + m->inc_ptr.bytes() + m->inc_elem.bytes() +
+                           m->order.bytes() + m->tiles.bytes();
+    return !m->arena.budget || pattern + plan + later_needs(m) <= m->arena.budget;
+}
+
+// The same of a plan with lists that is made: its buffers may have taken kept blocks larger
+// than they are.
+static bool budget_still_holds(fem_mesh m) {
+    const Plan &P = m->plan;
+    if (!m->arena.budget || !P.full.lists.ready) return true;
+    size_t held = m->ke64.bytes() + m->chunk_slots.bytes() + m->tiles.partial.bytes();
+    for (const auto &slot : m->host_stage) held += slot.bytes();
+    const size_t pos = P.full.celem_pos.ptr ? 0 : (size_t)P.full.total_celems * P.pos_stride;
+    return m->arena.live - held + pos + later_needs(m) <= m->arena.budget;
 }
 
 // Gather lists serve the scalar operators' builds; the fused FP64 form and the
@@ -1930,6 +1944,11 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
             continue;
         }
         if (st == PLAN_AGAIN) {
+            m->lists_off = true;
+            continue;
+        }
+        if (st == FEM_OK && !budget_still_holds(m)) {
+            m->xrank.free();
             m->lists_off = true;
             continue;
         }
