@@ -354,8 +354,6 @@ static PatchArgs patch_args(fem_mesh m, fem_prec p, bool fused) {
     a.threads = m->opt.block_threads > 0 ? m->opt.block_threads : 256;
     if (a.threads > patch_max_threads(m->npe)) a.threads = patch_max_threads(m->npe);
     a.threads = (a.threads + 31) / 32 * 32;
-    // assembling given element matrices, one block fills an SM's shared memory
-    if (!fused && m->opt.block_threads <= 0 && m->plan.full.lists.ready) a.threads = 512;
     if (is_elastic(m)) a.threads = elastic_threads(m->npe, m->opt.block_threads);  // its own default and cap
     a.blocks_per_sm = m->opt.blocks_per_sm;
     a.mode = kernel_mode(m->opt);
