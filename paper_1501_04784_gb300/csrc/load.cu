@@ -24,6 +24,35 @@ struct LoadSmem {
     size_t xs, cown, gid, fs, total;
 };
 
+template <typename S>
+struct TetX {
+    S x[4][3];
+};
+
+// |det J| of a tetrahedron.  One copy of the code: inlined, the compiler contracts it one
+// way in one kernel and another way in the next, and F is the same bit for bit with and
+// without gather lists.
+template <typename T, typename S, bool MIXED>
+__device__ __noinline__ T tet_abs_det(TetX<S> t, float thr, bool fp64_det) {
+    T det;
+    if constexpr (MIXED) {
+        Vec3<float> Fv[4];
+        float d;
+        tet_geometry_mixed<S>(t.x, thr, fp64_det, Fv, d);
+        det = d;
+    } else {
+        TetGeom<T> g;
+        tet_geom<T, S>(t.x, g);
+        Vec3<T> Fv[4];
+        tet_faces(g, Fv, det);
+    }
+    return det < T(0) ? -det : det;
+}
+
+// (a product that is not contracted into the sums either)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // Load vector of one element: s times the integrals of its shape functions.
 template <int NPE, typename T, typename S, bool MIXED>
 __device__ __forceinline__ void element_load(const S (*xc)[3], T s, float thr, bool fp64_det, T (&fe)[NPE]) {
@@ -32,19 +61,12 @@ __device__ __forceinline__ void element_load(const S (*xc)[3], T s, float thr, b
         brick_gauss_dets<T, S>(xc, thr, MIXED, det);
         brick_load_from_dets(det, s, fe);
     } else {
-        T det;
-        if constexpr (MIXED) {
-            Vec3<float> Fv[4];
-            float d;
-            tet_geometry_mixed<S>(xc, thr, fp64_det, Fv, d);
-            det = d;
-        } else {
-            TetGeom<T> g;
-            tet_geom<T, S>(xc, g);
-            Vec3<T> Fv[4];
-            tet_faces(g, Fv, det);
-        }
-        const T share = s * (det < T(0) ? -det : det) * T(1.0 / 24.0);
+        TetX<S> t;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) t.x[a][d] = xc[a][d];
+        const T share = mul_rn(mul_rn(s, tet_abs_det<T, S, MIXED>(t, thr, fp64_det)), T(1.0 / 24.0));
 #pragma unroll
         for (int a = 0; a < 4; ++a) fe[a] = share;
     }
@@ -209,9 +231,7 @@ template <int NPE, typename T, typename S, typename CT, bool MIXED, int NC>
 static fem_status launch_load_t(fem_mesh m, const Closure &cl, const void *X, const void *src, void *F, float thr,
                                 bool fp64_det, cudaStream_t s) {
     const Plan &P = m->plan;
-    // Tetrahedra keep the colour form: the compiler contracts their determinants
-    // differently in the two kernels, and F is the same bit for bit with and without lists.
-    if constexpr (NC == 1 && NPE == 8) {
+    if constexpr (NC == 1) {
         if (cl.lists.ready) {
             LoadListSmem L{};
             L.fe = al16((size_t)P.max_cnodes * 3 * sizeof(S));
