@@ -79,7 +79,11 @@ typedef enum { FEM_FP64 = 0, FEM_MIXED = 1 } fem_prec;
 typedef enum { FEM_F32 = 0, FEM_F64 = 1 } fem_dtype;
 
 typedef struct {
-    size_t mem_budget_bytes;     /* cap on library-owned device memory; 0 = no cap */
+    size_t mem_budget_bytes;     /* cap on library-owned device memory; 0 = no cap.  Under a cap
+                                    the gather lists of a plan (fem_info.gather_lists) give way
+                                    to what a call needs: the first call that finds no room
+                                    beside them makes the plan again without them and blocks
+                                    meanwhile (not once a call was captured) */
     double distortion_threshold; /* mixed mode; brick: max_q detJ / min_q detJ, tet:
                                     longest edge / shortest altitude.  0 = default
                                     (brick 4, tetrahedron 10). */

@@ -361,6 +361,56 @@ static PatchArgs patch_args(fem_mesh m, fem_prec p, bool fused) {
     return a;
 }
 
+// Under a budget, library memory that calls take as they need it must not decide how the
+// next plan is made: the FP64 matrices and the host builds' staging are given back (and
+// taken again by the calls that use them).
+static void make_room(fem_mesh m) {
+    if (!m->arena.budget) return;
+    cudaDeviceSynchronize();
+    m->ke64.free();
+    m->chunk_slots.free();
+    for (auto &slot : m->host_stage) slot.free();
+}
+
+static size_t missing(size_t want, size_t have) { return want > have ? want - have : 0; }
+
+// Library memory that a device build takes beyond what the mesh holds: the FP64 element
+// matrices, or the tiles' partial rows.
+static size_t build_needs(fem_mesh m, fem_prec p, bool tiles) {
+    if (tiles)
+        return missing((size_t)m->tiles.partial_n * (p == FEM_FP64 ? sizeof(double) : sizeof(float)),
+                       m->tiles.partial.bytes());
+    if (p != FEM_FP64 || m->opt.fp64_fused || m->plan.chunked) return 0;
+    return missing((size_t)m->n_elems * m->np * sizeof(double), m->ke64.bytes());
+}
+
+// Under a budget gather lists are taken where they fit, but they only make builds faster
+// (and the plan a fifth larger: 27M bricks 9.83 GB with them, 8.10 without), while the
+// memory a call needs decides whether it can run at all, or runs staged.  So a call that
+// finds no room for `need` bytes gets that of the lists: the ordered coordinates first,
+// then the plan is made again for the scatter, as it would have been without lists.  Not
+// under capture, and not once a call was captured: its graph reads the plan that is there.
+static fem_status ensure_room(fem_mesh m, size_t need, cudaStream_t s) {
+    const Arena &ar = m->arena;
+    if (!ar.budget) return FEM_OK;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        m->captured = true;
+    }
+    auto fits = [&] { return ar.live + need <= ar.budget; };
+    if (m->captured || !m->plan_built || !m->plan.full.lists.ready || fits()) return FEM_OK;
+    FEM_CUDA(cudaDeviceSynchronize());
+    m->xrank.free();
+    if (fits()) return FEM_OK;
+    make_room(m);
+    m->lists_denied = true;
+    m->plan_built = false;
+    FEM_TRY(build_plan(m, s));  // (no blocks kept: the plan's buffers are to be no larger than they need)
+    m->plan_built = true;
+    return FEM_OK;
+}
+
 fem_status fem_assemble_csr(fem_mesh m, fem_prec p, const void *ke, void *vals, void *stream) {
     if (!m) {
         set_error("null mesh");
@@ -381,6 +431,7 @@ fem_status fem_assemble_csr(fem_mesh m, fem_prec p, const void *ke, void *vals, 
     }
     cudaStream_t s = as_stream(stream);
     FEM_TRY(ensure_plan(m, s));
+    FEM_TRY(ensure_room(m, 0, s));
     PatchArgs a = patch_args(m, p, false);
     a.xd = FEM_F32;
     a.cd = FEM_F32;
@@ -393,8 +444,8 @@ fem_status fem_assemble_csr(fem_mesh m, fem_prec p, const void *ke, void *vals, 
     });
 }
 
-fem_status fem_build_K(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype, const void *c, fem_dtype c_dtype,
-                       void *vals, void *stream) {
+static fem_status build_K(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype, const void *c, fem_dtype c_dtype,
+                          void *vals, void *stream, bool room) {
     NvtxRange nvtx_range("fem_build_K");
     FEM_TRY(check_inputs(m, p, X, x_dtype, c, c_dtype));
     if (!m->has_pattern) {
@@ -406,6 +457,7 @@ fem_status fem_build_K(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype,
         return FEM_ERR_ARG;
     }
     cudaStream_t s = as_stream(stream);
+    if (room && use_tiles(m)) FEM_TRY(ensure_room(m, build_needs(m, p, true), s));
     if (use_tiles(m)) {
         // element tiles: each element integrated once, in the build's precision
         TilePlan &T = m->tiles;
@@ -439,6 +491,7 @@ fem_status fem_build_K(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype,
         cudaGetLastError();  // no room for the partials: patches
     }
     FEM_TRY(ensure_plan(m, s));
+    if (room) FEM_TRY(ensure_room(m, build_needs(m, p, false), s));
     if (is_elastic(m)) {
         if (p == FEM_FP64 && m->opt.fp64_fused == 0) {
             // FP64 integrates each element once into library memory (300 or 78
@@ -511,6 +564,11 @@ fem_status fem_build_K(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype,
     });
 }
 
+fem_status fem_build_K(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype, const void *c, fem_dtype c_dtype,
+                       void *vals, void *stream) {
+    return build_K(m, p, X, x_dtype, c, c_dtype, vals, stream, true);
+}
+
 namespace fem {
 // Device address of a page-locked host buffer (unified addressing), or null if
 // the buffer is not page-locked.
@@ -523,6 +581,11 @@ static void *mapped(void *host) {
     return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+// One of the host pipeline's two slots: the values of the largest row range.
+static size_t chunk_slot_bytes(fem_mesh m, fem_prec p) {
+    return ((size_t)m->plan.max_chunk_vals * (p == FEM_FP64 ? sizeof(double) : sizeof(float)) + 255) / 256 * 256;
+}
+
 // Host pipeline over the plan's row ranges (fem_options.host_chunks): range k is
 // built into device slot k % 2 on s while the values of range k - 1 go from the
 // other slot to vals_host on the mesh's copy stream (Section 4.3: one group's
@@ -532,7 +595,7 @@ static fem_status chunk_pipeline(fem_mesh m, fem_prec p, const void *X, fem_dtyp
                                  void *vals_host, cudaStream_t s) {
     Plan &P = m->plan;
     const size_t w = p == FEM_FP64 ? sizeof(double) : sizeof(float);
-    const size_t slot = ((size_t)P.max_chunk_vals * w + 255) / 256 * 256;
+    const size_t slot = chunk_slot_bytes(m, p);
     if (!m->copy_stream) FEM_CUDA(cudaStreamCreateWithFlags(&m->copy_stream, cudaStreamNonBlocking));
     for (int j = 0; j < 2; ++j) {
         if (!m->chunk_built[j]) FEM_CUDA(cudaEventCreateWithFlags(&m->chunk_built[j], cudaEventDisableTiming));
@@ -630,6 +693,9 @@ static fem_status host_build(fem_mesh m, fem_prec p, const void *X_host, fem_dty
         FEM_TRY(ensure_plan(m, s));
         pipe = m->plan.n_chunks() > 1;
     }
+    const bool staged = !pipe && !m->opt.host_direct;
+    FEM_TRY(ensure_room(m, missing(staged ? vo + vb : vo, m->host_stage[k].bytes()) + build_needs(m, p, use_tiles(m)) +
+                               (pipe ? missing(chunk_slot_bytes(m, p) * 2, m->chunk_slots.bytes()) : 0), s));
     const bool stage_fits = pipe || m->host_stage[k].n >= vo + vb || !m->arena.budget ||
                             m->arena.live - m->host_stage[k].n + vo + vb <= m->arena.budget;
     if (m->opt.host_direct || !stage_fits) {
@@ -658,7 +724,7 @@ static fem_status host_build(fem_mesh m, fem_prec p, const void *X_host, fem_dty
     if (pipe)
         FEM_TRY(chunk_pipeline(m, p, base + xo, x_dtype, base + co, c_dtype, vals_host, s));
     else
-        FEM_TRY(fem_build_K(m, p, base + xo, x_dtype, base + co, c_dtype, direct ? direct : base + vo, s));
+        FEM_TRY(build_K(m, p, base + xo, x_dtype, base + co, c_dtype, direct ? direct : base + vo, s, false));
     FEM_CUDA(cudaEventRecord(m->built, s));
     if (!direct && !pipe) FEM_CUDA(cudaMemcpyAsync(vals_host, base + vo, vb, cudaMemcpyDeviceToHost, s));
     FEM_CUDA(cudaEventRecord(m->stage_free[k], s));
@@ -707,6 +773,11 @@ fem_status fem_vjp(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype, con
         return FEM_ERR_ARG;
     }
     FEM_TRY(ensure_plan(m, as_stream(stream)));
+    // the first pass adds the in-row positions; the gradients of every element are staged
+    const Closure &cl = m->plan.full;
+    FEM_TRY(ensure_room(m, (cl.celem_pos.ptr ? 0 : (size_t)cl.total_celems * m->plan.pos_stride) +
+                               (m->opt.vjp_fused ? 0 : missing((size_t)m->n_elems * m->npe * 3 * w, m->ke64.bytes())),
+                        as_stream(stream)));
     FEM_TRY(ensure_positions(m, as_stream(stream)));
     if (is_elastic(m))
         return launch_elastic_vjp(m, p == FEM_MIXED, X, x_dtype, c, c_dtype, G, dX, dc, as_stream(stream));
@@ -726,6 +797,7 @@ fem_status fem_load_vector(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dt
         return FEM_ERR_ARG;
     }
     FEM_TRY(ensure_plan(m, as_stream(stream)));
+    FEM_TRY(ensure_room(m, 0, as_stream(stream)));
     return launch_load(m, p == FEM_MIXED, X, x_dtype, src, src_dtype, F, default_threshold(m), m->opt.fp64_dets != 0,
                        as_stream(stream));
 }
@@ -789,17 +861,6 @@ fem_status fem_batched_config(const fem_mesh *meshes, int n, fem_prec p, int *bl
     return batched_query(meshes, n, p == FEM_MIXED, block_threads, blocks_per_sm, grid);
 }
 
-// Under a budget, library memory that calls take as they need it must not decide how the
-// next plan is made: the FP64 matrices and the host builds' staging are given back (and
-// taken again by the calls that use them).
-static void make_room(fem_mesh m) {
-    if (!m->arena.budget) return;
-    cudaDeviceSynchronize();
-    m->ke64.free();
-    m->chunk_slots.free();
-    for (auto &slot : m->host_stage) slot.free();
-}
-
 // Tuner of the assembly tile and of the threads per block: the plan is rebuilt
 // for each candidate size (elements per tile when the builds run on tiles,
 // lower-CSR entries per patch otherwise) and every candidate is timed on the
@@ -832,6 +893,7 @@ fem_status fem_autotune(fem_mesh m, fem_prec p, const void *X, fem_dtype x_dtype
     const size_t flush_bytes = (size_t)256 << 20;
     auto replan = [&](cudaStream_t st) -> fem_status {
         make_room(m);
+        m->lists_denied = false;
         if (m->arena.budget) flush.free();
         if (tiles) return build_tiles(m, st);
         fem_status r = build_plan(m, st);
@@ -920,6 +982,7 @@ fem_status fem_set_tuning(fem_mesh m, int patch_entries, int block_threads, void
     if (!m->has_pattern) return FEM_OK;  // fem_pattern will plan with these settings
     cudaStream_t s = as_stream(stream);
     make_room(m);
+    m->lists_denied = false;
     ArenaKeep keep(m->arena);
     fem_status st = FEM_OK;
     if (use_tiles(m)) {

@@ -336,16 +336,6 @@ fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s) {
     const int64_t np_ = cl.p1 - cl.p0;
     const int np = m->npe * (m->npe + 1) / 2;
     G.zero = (int)(cl.max_celems * np);
-    // Under a budget, beside everything the calls may take later (the first backward pass
-    // adds the in-row positions to the plan).
-    auto room = [&](size_t n_words) {
-        size_t plan = P.bytes() + n_words * sizeof(uint32_t);
-        if (!cl.celem_pos.ptr) plan += (size_t)cl.total_celems * P.pos_stride;
-        if (wants_ordered_x(m)) plan += 4 * sizeof(float) * (size_t)m->n_nodes;
-        if (budget_holds(m, plan)) return true;
-        set_error("memory budget: no room for gather lists");
-        return false;
-    };
     FEM_TRY(G.patch.alloc(m->arena, np_, "gather patches"));
     DevBuf<unsigned long long> cursor;
     FEM_TRY(cursor.alloc(m->arena, 2, "gather list cursor"));
@@ -359,7 +349,6 @@ fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s) {
     auto f = m->npe == 8 ? k_gather_lists<8> : k_gather_lists<4>;
     FEM_CUDA(allow_smem(f, L.total));
     for (int pass = 0; pass < 2; ++pass) {
-        if (!room(cap)) return FEM_ERR_BUDGET;
         FEM_TRY(G.words.alloc(m->arena, cap, "gather lists"));
         FEM_CUDA(cudaMemsetAsync(cursor.ptr, 0, 2 * sizeof(unsigned long long), s));
         f<<<grid, 512, L.total, s>>>(P.view(cl), m->col.ptr, L, top_step, (uint32_t)G.zero, G.patch.ptr, G.words.ptr, cursor.ptr,

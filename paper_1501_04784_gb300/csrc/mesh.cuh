@@ -235,6 +235,8 @@ struct fem_mesh_s {
     bool plan_built = false;  // the patch plan exists (it is built on first use when tiles serve the builds)
     bool lone_node = false;   // a node has no element: gather lists hold a diagonal for every row
     bool lists_off = false;   // the present plan was made without gather lists (decided anew by each plan)
+    bool lists_denied = false;  // under the budget the calls needed the lists' room (until the next tuning)
+    bool captured = false;      // a call was captured (noted under a budget): its graph reads the plan
     bool want_pos = false;    // closures carry the in-row positions (set by the first backward pass)
     fem::TilePlan tiles;      // element tiles of the scalar operators (tile.cuh)
     // device status word: set by a bounded device-side wait that gave up
@@ -308,9 +310,7 @@ constexpr fem_status PLAN_AGAIN = static_cast<fem_status>(1000);
 // Gather lists of a closure (gather_plan.cu), and whether mesh m's builds may run on them.
 fem_status build_gather_lists(fem_mesh m, Closure &cl, cudaStream_t s);
 bool wants_lists(fem_mesh m);
-// Whether the budget holds the pattern and `plan` bytes beside what the calls may take later.
-bool budget_holds(fem_mesh m, size_t plan);
-// Nodes from which single meshes' FP32 coordinates are put in locality order (symbolic.cu).
+// Whether the plan's FP32 coordinates are put in locality order first (symbolic.cu).
 bool wants_ordered_x(fem_mesh m);
 // One call's use of the mesh's ordered coordinates.  A mixed build writes nothing of the
 // mesh's but its status word, and calls on several streams or threads rely on that, so

@@ -1632,38 +1632,6 @@ fem_status build_closure(fem_mesh m, int64_t p0, int64_t p1, Closure &cl, cudaSt
 
 bool wants_ordered_x(fem_mesh m) { return m->n_nodes >= XRANK_MIN && !m->plan.id_runs; }
 
-// Lists are about a fifth of a plan (27M bricks: 9.83 GB with them, 8.10 without) and only
-// make builds faster; the library memory that calls take as they need it decides whether
-// they can run, or whether FP64 builds and backward passes run staged.  So under a budget
-// lists are taken only where all of that fits beside them: the FP64 element matrices (or
-// the backward's element gradients, in the same buffer), the host builds' three staging
-// slots, the tiles' partial rows, the tuner's scratch.  It depends on the mesh and the
-// budget alone, not on what is held when a plan is made.
-static size_t later_needs(fem_mesh m) {
-    const size_t N = (size_t)m->n_nodes, nel = (size_t)m->n_elems, nnz = (size_t)m->nnz;
-    const size_t staged = nel * (size_t)std::max(m->np, 3 * m->npe) * sizeof(double);
-    const size_t host = fem_mesh_s::HOST_STAGES * (24 * N + 8 * nel + 8 * nnz + 1024);
-    const size_t partial = m->tiles.ready ? (size_t)m->tiles.partial_n * sizeof(double) : 0;
-    return staged + host + partial + ((size_t)256 << 20);
-}
-
-bool budget_holds(fem_mesh m, size_t plan) {
-    const size_t pattern = m->rowptr.bytes() + m->col.bytes() + m->inc_ptr.bytes() + m->inc_elem.bytes() +
-                           m->order.bytes() + m->tiles.bytes();
-    return !m->arena.budget || pattern + plan + later_needs(m) <= m->arena.budget;
-}
-
-// The same of a plan with lists that is made: its buffers may have taken kept blocks larger
-// than they are.
-static bool budget_still_holds(fem_mesh m) {
-    const Plan &P = m->plan;
-    if (!m->arena.budget || !P.full.lists.ready) return true;
-    size_t held = m->ke64.bytes() + m->chunk_slots.bytes() + m->tiles.partial.bytes();
-    for (const auto &slot : m->host_stage) held += slot.bytes();
-    const size_t pos = P.full.celem_pos.ptr ? 0 : (size_t)P.full.total_celems * P.pos_stride;
-    return m->arena.live - held + pos + later_needs(m) <= m->arena.budget;
-}
-
 // Gather lists serve the scalar operators' builds; the fused FP64 form and the
 // test of the phase waits run on the colour-ordered scatter.
 bool wants_lists(fem_mesh m) {
@@ -1929,7 +1897,16 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
     // another stream may still run on the plan that goes: its ranges are used again here
     if (m->plan.n_patches > 0) FEM_CUDA(cudaDeviceSynchronize());
     m->xrank.free();  // the new plan has its own, if any
-    m->lists_off = !budget_holds(m, 0);
+    m->lists_off = m->lists_denied;
+    // (under a budget released blocks are no longer kept for the plan that follows: its
+    // buffers would take ones up to twice their size, and the calls' staging lack them)
+    auto without_lists = [m] {
+        m->lists_off = true;
+        if (!m->arena.budget) return;
+        m->arena.keep = false;
+        m->plan.reset();
+        m->arena.trim();
+    };
     int64_t cap = 0;
     for (;;) {
         const fem_status st = build_plan_cap(m, s, cap);
@@ -1940,16 +1917,11 @@ fem_status build_plan(fem_mesh m, cudaStream_t s) {
         if (cap == 0 && (st == FEM_OK || st == FEM_ERR_BUDGET) && wants_lists(m) && !m->plan.full.lists.ready &&
             default_list_patches(m)) {
             cudaGetLastError();
-            m->lists_off = true;
+            without_lists();
             continue;
         }
         if (st == PLAN_AGAIN) {
-            m->lists_off = true;
-            continue;
-        }
-        if (st == FEM_OK && !budget_still_holds(m)) {
-            m->xrank.free();
-            m->lists_off = true;
+            without_lists();
             continue;
         }
         FEM_TRY(st);

@@ -89,19 +89,43 @@ def test_ordered_coordinates_under_a_budget(fem):
     G = torch.randn(free.nnz, device="cuda", generator=torch.Generator("cuda").manual_seed(5))
     dX, dc = free.vjp(X, c, G, "mixed")
     plain.vjp(X, c, G, "mixed")
-    lists, scatter = free.info()["n_patches"], plain.info()["n_patches"]
-    assert lists > scatter
+    assert free.info()["gather_lists"] == 1 and plain.info()["gather_lists"] == 0
     seen = set()
     for extra in (0, 4, 16, 64, 1024):
         budget = plain.info()["peak_bytes"] + extra * MB
         mesh = fem.Mesh(E, m.n_nodes, X=X, mem_budget_bytes=budget)
         v = mesh.build_K(X, c, "mixed")
-        planned = mesh.info()["n_patches"]
         assert float((v - want).abs().max()) <= 4e-6 * float(want.abs().max())
         for u, w in zip(mesh.vjp(X, c, G, "mixed"), (dX, dc)):
             assert float((u - w).abs().max()) <= 4e-6 * float(w.abs().max())
+        fem.launch_count(reset=True)
+        mesh.vjp(X, c, G, "mixed")
+        assert fem.launch_count() in (2, 3)  # staged, the coordinates ordered or not
         info = mesh.info()
-        assert info["n_groups"] == 1 and info["n_patches"] == planned and info["peak_bytes"] <= budget
-        seen.add(planned)
+        assert info["n_groups"] == 1 and info["peak_bytes"] <= budget
+        seen.add(info["gather_lists"])
         mesh.sync()
-    assert seen == {lists, scatter}
+    assert seen == {0, 1}
+
+
+def test_captured_calls_keep_their_plan(fem, case):
+    """A captured build reads the plan it was captured with: calls that would need the
+    lists' room afterwards do without."""
+    m, E, X, c = case
+    free = fem.Mesh(E, m.n_nodes, X=X, mem_budget_bytes=1 << 40)
+    want = free.build_K(X, c, "mixed").clone()
+    mesh = fem.Mesh(E, m.n_nodes, X=X, mem_budget_bytes=free.info()["peak_bytes"] + MB)
+    out = torch.zeros_like(want)
+    assert torch.equal(mesh.build_K(X, c, "mixed"), want) and mesh.info()["gather_lists"] == 1
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        mesh.build_K(X, c, "mixed", out=out)
+    a = mesh.build_K(X.double(), c.double(), "fp64")  # 18 MB of matrices: fused instead
+    b = free.build_K(X.double(), c.double(), "fp64")
+    assert float((a - b).abs().max()) <= 1.6e-13 * float(b.abs().max())
+    assert mesh.info()["gather_lists"] == 1
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want)
+    mesh.sync()
