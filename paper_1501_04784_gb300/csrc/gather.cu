@@ -16,9 +16,9 @@
 // summed, cp.async brings the next patch's coordinates and coefficients.  Patches are
 // smaller than the scatter's (the matrices of 500 bricks fill half an SM's shared
 // memory), so more border elements are integrated twice; on balance 1M bricks went
-// from 228 to 171 us, 27M from 4.87 to 3.88 ms, 512 meshes in one launch from 3.17 to
-// 2.70 ms, 3.07M tetrahedra from 160 to 152 us, and the assembly of 1M bricks' FP64
-// matrices from 0.36 to 0.29 ms.  What bounds it now: latency at 16 warps an SM (110
+// from 228 to 167 us, 27M from 4.87 to 3.75 ms, 512 meshes in one launch from 3.17 to
+// 2.66 ms, 3.07M tetrahedra from 160 to 146 us, and the assembly of 1M bricks' FP64
+// matrices from 0.36 to 0.28 ms.  What bounds it now: latency at 16 warps an SM (113
 // registers; 20 or 24 warps at 96 or 80 registers measured slower), about two thirds
 // of it in the integration.
 #include "elem_ops.cuh"
