@@ -157,7 +157,9 @@ struct LoadListSmem {
 
 template <int NPE, typename T, typename S, typename CT, bool MIXED>
 __global__ void __launch_bounds__(256) k_load_lists(PlanView pv, const S *__restrict__ X, const CT *__restrict__ src,
-                                                    T *__restrict__ F, float thr, bool fp64_det, LoadListSmem L) {
+                                                    T *__restrict__ F, float thr, bool fp64_det, LoadListSmem L,
+                                                    int *status) {
+    (void)status;  // (bounds-check build)
     constexpr int NP = NPE * (NPE + 1) / 2;
     extern __shared__ __align__(16) unsigned char ll_smem[];
     S(*xs)[3] = reinterpret_cast<S(*)[3]>(ll_smem + L.xs);
@@ -172,6 +174,7 @@ __global__ void __launch_bounds__(256) k_load_lists(PlanView pv, const S *__rest
             for (int u = 0; u < CH; ++u) {
                 const int j = j0 + u * nthr;
                 g[u] = j < d.n_cnodes ? __ldg(pv.cnode_gid + d.cb + j) : 0;
+                if (!FEM_IN_BOUNDS(g[u] >= 0 && g[u] < pv.n_nodes, status)) g[u] = 0;
             }
             S v[CH][3];
 #pragma unroll
@@ -186,9 +189,14 @@ __global__ void __launch_bounds__(256) k_load_lists(PlanView pv, const S *__rest
         }
         __syncthreads();
         for (int i = tid; i < d.n_elems; i += nthr) {
-            const T s = (T)__ldg(src + __ldg(pv.celem_id + d.eb + i));
+            int64_t e = __ldg(pv.celem_id + d.eb + i);
+            if (!FEM_IN_BOUNDS(e >= 0 && e < pv.n_elems, status)) e = 0;
+            const T s = (T)__ldg(src + e);
             uint16_t ln[NPE];
             load_lnodes<NPE>(pv.celem_lnode, d.eb + i, ln);
+#pragma unroll
+            for (int a = 0; a < NPE; ++a)
+                if (!FEM_IN_BOUNDS(ln[a] < d.n_cnodes, status)) ln[a] = 0;
             S xc[NPE][3];
 #pragma unroll
             for (int a = 0; a < NPE; ++a) xc[a][0] = xs[ln[a]][0], xc[a][1] = xs[ln[a]][1], xc[a][2] = xs[ln[a]][2];
@@ -204,7 +212,7 @@ __global__ void __launch_bounds__(256) k_load_lists(PlanView pv, const S *__rest
             const uint4 t = __ldg(tab + ch);
             T s = T(0);
             auto add = [&](uint32_t q) {
-                if ((int)q == pv.gzero) return;
+                if ((int)q == pv.gzero || !FEM_IN_BOUNDS((int)q < d.n_elems * NP, status)) return;
                 // packed diagonal entry a (a + 3) / 2 of element q / NP
                 const uint32_t i = q / NP, r = q - i * NP;
                 int a = 0;
@@ -219,7 +227,10 @@ __global__ void __launch_bounds__(256) k_load_lists(PlanView pv, const S *__rest
                 add(q >> 16);
             }
             const int k = 32 * ch + lane;
-            if (k < d.n_own) F[pv.own_row[d.nb + k]] = s;
+            if (k < d.n_own) {
+                const int64_t r = pv.own_row[d.nb + k];
+                if (FEM_IN_BOUNDS(r >= 0 && r < pv.n_nodes, status)) F[r] = s;
+            }
         }
         __syncthreads();
     }
@@ -243,7 +254,8 @@ static fem_status launch_load_t(fem_mesh m, const Closure &cl, const void *X, co
             const int64_t np = cl.p1 - cl.p0;
             if (np <= 0) return FEM_OK;
             const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(np, (int64_t)num_sms() * std::max(per_sm, 1)));
-            f<<<grid, 256, L.total, s>>>(P.view(cl), (const S *)X, (const CT *)src, (T *)F, thr, fp64_det, L);
+            f<<<grid, 256, L.total, s>>>(P.view(cl), (const S *)X, (const CT *)src, (T *)F, thr, fp64_det, L,
+                                      m->status.ptr);
             FEM_LAUNCHED("k_load_lists");
             return FEM_OK;
         }

@@ -858,7 +858,8 @@ struct SumSmem {
 
 template <int NPE, typename T>
 __global__ void __launch_bounds__(256) k_vjp_sum(PlanView pv, const T *__restrict__ dxe, T *__restrict__ dX,
-                                                 SumSmem L) {
+                                                 SumSmem L, int *status) {
+    (void)status;  // (bounds-check build)
     constexpr int NP = NPE * (NPE + 1) / 2, R = NPE * 3, Q = R * (int)sizeof(T) / 16;  // 16-byte pieces of a row
     extern __shared__ __align__(16) unsigned char vs_smem[];
     T *dx = reinterpret_cast<T *>(vs_smem + L.dx);
@@ -867,7 +868,8 @@ __global__ void __launch_bounds__(256) k_vjp_sum(PlanView pv, const T *__restric
     for (int64_t p = blockIdx.x; p < pv.n_patches; p += gridDim.x) {
         const GatherPatch d = pv.gpatch[p];
         for (int t = tid; t < d.n_elems * Q; t += nthr) {
-            const int64_t e = __ldg(pv.celem_id + d.eb + t / Q);
+            int64_t e = __ldg(pv.celem_id + d.eb + t / Q);
+            if (!FEM_IN_BOUNDS(e >= 0 && e < pv.n_elems, status)) e = 0;
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dx) + 16 * t),
                          "l"(reinterpret_cast<const unsigned char *>(dxe) + (e * Q + t % Q) * 16)
                          : "memory");
@@ -880,7 +882,7 @@ __global__ void __launch_bounds__(256) k_vjp_sum(PlanView pv, const T *__restric
             const uint4 t = __ldg(tab + ch);
             T s[3] = {T(0), T(0), T(0)};
             auto add = [&](uint32_t q) {
-                if ((int)q == pv.gzero) return;
+                if ((int)q == pv.gzero || !FEM_IN_BOUNDS((int)q < d.n_elems * NP, status)) return;
                 // packed diagonal entry a (a + 3) / 2 of element q / NP
                 const uint32_t i = q / NP, r = q - i * NP;
                 int a = 0;
@@ -901,7 +903,8 @@ __global__ void __launch_bounds__(256) k_vjp_sum(PlanView pv, const T *__restric
         __syncthreads();
         for (int t = tid; t < 3 * d.n_own; t += nthr) {
             const int k = t / 3;
-            dX[3 * (int64_t)__ldg(pv.own_row + d.nb + k) + (t - 3 * k)] = out[t];
+            const int64_t r = __ldg(pv.own_row + d.nb + k);
+            if (FEM_IN_BOUNDS(r >= 0 && r < pv.n_nodes, status)) dX[3 * r + (t - 3 * k)] = out[t];
         }
         __syncthreads();
     }
@@ -945,7 +948,7 @@ static fem_status launch_vjp_sum_t(fem_mesh m, const Closure &cl, const void *dx
     fem_status st;
     const int grid = grid_for((const void *)f, 256, L.total, cl.p1 - cl.p0, "backward sum kernel", &st);
     if (st != FEM_OK) return st;
-    f<<<grid, 256, L.total, s>>>(m->plan.view(cl), (const T *)dxe, (T *)dX, L);
+    f<<<grid, 256, L.total, s>>>(m->plan.view(cl), (const T *)dxe, (T *)dX, L, m->status.ptr);
     FEM_LAUNCHED("k_vjp_sum");
     return FEM_OK;
 }
